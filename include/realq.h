@@ -535,13 +535,14 @@ realq_status_t realq_set_tensor_overlap(int mode);
 realq_status_t realq_set_block_attention(int mode);
 
 /* Tuning: the products of the block ops (realq_block_*, and the window
- * quantization's loss).  0 (default): fp32 CUDA-core tiles for all; 1:
- * tf32x3 tensor-core products where the operands fit the workspace's plane
- * scratch.  tf32x3 keeps 22 significant bits of each operand against fp32's
- * 24, and the window's loss (a difference of two forward passes) magnifies
- * that about tenfold: its gradient moves a few group scales of a window
- * sweep by more than 1e-5, while the projections are under 1 % of the
- * window's time (the attention is the rest).
+ * quantization's loss).  0 (default): fp32 accuracy: bf16x6 tensor-core
+ * products (three bf16 planes per operand, all 24 significant bits, sums
+ * promoted to fp32 registers every 32 terms) from 64 x 64 outputs and K = 64
+ * on where the operands fit the workspace's plane scratch, fp32 CUDA-core
+ * tiles otherwise; 1: tf32x3 tensor-core products.  tf32x3 keeps 22
+ * significant bits of each operand, and the window's loss (a difference of
+ * two forward passes) magnifies that about tenfold: its gradient moves a few
+ * group scales of a window sweep by more than 1e-5.
  * Process-wide.  REALQ_ERR_INVALID_ARG for other values.  No counterpart in
  * the paper. */
 realq_status_t realq_set_block_products(int mode);
@@ -585,9 +586,8 @@ realq_status_t realq_reverse_cosine_lr(int64_t i, int64_t L, double lr_final, do
  *             first int is a status word that each call clears at its start
  *             and that a timed-out bounded wait of a tensor-core product
  *             sets (read it with realq_workspace_status).
- * Computed in fp32 with fp32 accumulation (the loss summed in double); with
- * realq_set_block_products(1) the projections and products whose operands
- * fit the workspace's plane scratch run as tf32x3 tensor-core products.
+ * Computed in fp32 with fp32 accumulation (the loss summed in double);
+ * realq_set_block_products selects how the projections and products run.
  * Asynchronous on `stream`; argument errors are returned before any launch.
  * S L is at most 4194240 tokens.  Outputs may not alias inputs. */
 typedef struct {

@@ -682,8 +682,9 @@ def realq_set_block_attention(mode: int) -> None:
 
 
 def realq_set_block_products(mode: int) -> None:
-    """Products of the block ops: 0 fp32 CUDA-core tiles (default), 1 tf32x3
-    tensor cores where the operands fit the workspace's plane scratch."""
+    """Products of the block ops: 0 fp32 accuracy (default; bf16x6 tensor
+    cores from 64 x 64 x 64 on, CUDA-core tiles below), 1 tf32x3 tensor cores
+    where the operands fit the workspace's plane scratch."""
     _check(lib().realq_set_block_products(int(mode)))
 
 

@@ -16,38 +16,151 @@ __global__ void __launch_bounds__(256) map_kernel(int64_t count, Fn fn) {
     if (i < count) fn(i);
 }
 
+// The row passes of block_ops.cuh (RMSNorm and its backward, the loss's row
+// products), one warp per token: the bodies walk a row with one thread, whose
+// loads of consecutive threads lie a row apart (0.46 ms per RMSNorm of 4096
+// x 1024, against 12 us of DRAM time); here the lanes of a warp share a row,
+// each summing every 32nd element, and combine in a fixed butterfly.
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+__global__ void __launch_bounds__(256) rms_fwd_kernel(int64_t rows, blk::RmsFwd f) {
+    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (t >= rows) return;
+    const float *xr = f.x + t * f.d;
+    float ss = 0.f;
+    for (int64_t k = lane; k < f.d; k += 32) ss += xr[k] * xr[k];
+    ss = warp_sum(ss);
+    const float rr = 1.f / sqrtf(ss / (float)f.d + f.eps);
+    if (lane == 0) f.r[t] = rr;
+    float *yr = f.y + t * f.d;
+    for (int64_t k = lane; k < f.d; k += 32) yr[k] = xr[k] * rr * f.g[k];
+}
+
+__global__ void __launch_bounds__(256) rms_bwd_kernel(int64_t rows, blk::RmsBwd f) {
+    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (t >= rows) return;
+    const float *xr = f.x + t * f.d, *gr = f.gy + t * f.d;
+    const float rr = f.r[t];
+    float dot = 0.f;
+    for (int64_t k = lane; k < f.d; k += 32) dot += gr[k] * f.g[k] * xr[k];
+    dot = warp_sum(dot);
+    const float c = rr * rr * rr * dot / (float)f.d;
+    float *o = f.gx + t * f.d;
+    const float *br = f.base ? f.base + t * f.d : nullptr;
+    for (int64_t k = lane; k < f.d; k += 32) {
+        const float v = gr[k] * f.g[k] * rr - xr[k] * c;
+        o[k] = br ? br[k] + v : v;
+    }
+}
+
+__global__ void __launch_bounds__(256) row_dot_kernel(int64_t rows, blk::RowDot f) {
+    const int64_t t = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int lane = threadIdx.x & 31;
+    if (t >= rows) return;
+    const float *ar = f.a + t * f.d, *br = f.b + t * f.d;
+    float s = 0.f;
+    for (int64_t k = lane; k < f.d; k += 32) s += ar[k] * br[k];
+    s = warp_sum(s);
+    if (lane == 0) f.out[t] = s;
+}
+
+// one warp per chunk of kChunk values (lanes in double, fixed butterfly)
+__global__ void __launch_bounds__(32) chunk_sum_kernel(blk::ChunkSum f) {
+    const int64_t c = blockIdx.x;
+    const int64_t end = (c + 1) * blk::kChunk < f.count ? (c + 1) * blk::kChunk : f.count;
+    double acc = 0.0;
+    for (int64_t t = c * blk::kChunk + threadIdx.x; t < end; t += 32) acc += (double)f.rows[t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (threadIdx.x == 0) f.part[c] = acc;
+}
+
+// out[j * rows + i] = in[i * cols + j], 32 x 32 tiles through shared memory
+// (the flat body reads one column per warp)
+__global__ void __launch_bounds__(256) transpose_kernel(blk::Transpose f, int64_t tiles_c) {
+    __shared__ float tile[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t r0 = (blockIdx.x / tiles_c) * 32, c0 = (blockIdx.x % tiles_c) * 32;
+#pragma unroll
+    for (int q = 0; q < 32; q += 8)
+        if (r0 + ty + q < f.rows && c0 + tx < f.cols) tile[ty + q][tx] = f.in[(r0 + ty + q) * f.cols + c0 + tx];
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 32; q += 8)
+        if (c0 + ty + q < f.cols && r0 + tx < f.rows) f.out[(c0 + ty + q) * f.rows + r0 + tx] = tile[tx][ty + q];
+}
+
 int g_attn_tiled = 1;   // realq_set_block_attention
 
 // Each step returns nonzero once a launch has failed; the first failure's
-// status is kept and nothing more is launched.  With plane scratch (planes:
-// four buffers of cap floats) the projections whose shapes the tensor-core
-// path takes run as tf32x3 products on tcgen05: the operands are split into
-// K-major tf32 hi / lo planes (transposed where stored the other way) and
-// C = alpha A B + R is formed in the product's epilogue; the others, and
-// every product without scratch, run on the fp32 CUDA-core tiles.
+// status is kept and nothing more is launched.  The products run on tcgen05
+// where their operands fit the plane scratch (four buffers of cap floats):
+// the operands are split into K-major planes (transposed where stored the
+// other way) and C = alpha A B + R is formed in the product's epilogue; by
+// default three bf16 planes each (bf16x6: fp32 accuracy, gemm_x6.cu), with
+// tf32 set two tf32 planes (tf32x3).  The others run on the fp32 CUDA-core
+// tiles.
 struct DevExec {
     cudaStream_t s;
     float *planes = nullptr;
     size_t cap = 0;
     int *err = nullptr;   // status word of the products' bounded waits
     realq_status_t st = REALQ_OK;
+    bool tf32 = false;    // realq_set_block_products(1)
+
+    // bf16x6 from 64 x 64 outputs and K = 64 on: below that a product is one
+    // CTA's few microseconds either way and the split pass would dominate
+    bool x6_ok(const blk::Gemm &g) const {
+        const int64_t ldk = (g.K + 7) / 8 * 8;
+        return planes && !tf32 && g.M >= 64 && g.N >= 64 && g.K >= 64 && (size_t)std::max(g.M, g.N) * ldk * 3 <= 4 * cap &&
+               g.M < (1ll << 31) && g.N < (1ll << 31) && g.K < (1ll << 31);
+    }
 
     bool tc_ok(const blk::Gemm &g) const {
-        return planes && g.M >= 32 && g.N >= 32 && g.M % 4 == 0 && g.N % 4 == 0 && g.K >= 32 && g.K % 4 == 0 &&
+        return planes && tf32 && g.M >= 32 && g.N >= 32 && g.M % 4 == 0 && g.N % 4 == 0 && g.K >= 32 && g.K % 4 == 0 &&
                (size_t)g.M * g.K <= cap && (size_t)g.N * g.K <= cap && g.M < (1ll << 31) && g.N < (1ll << 31) &&
                g.K < (1ll << 31);
     }
 
-    template <class Fn>
-    int map(int64_t count, const Fn &fn, const char *name) {
+    template <class Launcher>
+    int launch(int64_t count, const char *name, const Launcher &go) {
         if (st != REALQ_OK) return 1;
         if (count <= 0) return 0;
         {
             Launch L(name, s);
-            map_kernel<<<(unsigned)ceil_div(count, 256), 256, 0, s>>>(count, fn);
+            go();
         }
         st = check_launch(name);
         return st != REALQ_OK;
+    }
+
+    template <class Fn>
+    int map(int64_t count, const Fn &fn, const char *name) {
+        return launch(count, name, [&] { map_kernel<<<(unsigned)ceil_div(count, 256), 256, 0, s>>>(count, fn); });
+    }
+
+    int map(int64_t count, const blk::RmsFwd &f, const char *name) {
+        return launch(count, name, [&] { rms_fwd_kernel<<<(unsigned)ceil_div(count, 8), 256, 0, s>>>(count, f); });
+    }
+    int map(int64_t count, const blk::RmsBwd &f, const char *name) {
+        return launch(count, name, [&] { rms_bwd_kernel<<<(unsigned)ceil_div(count, 8), 256, 0, s>>>(count, f); });
+    }
+    int map(int64_t count, const blk::RowDot &f, const char *name) {
+        return launch(count, name, [&] { row_dot_kernel<<<(unsigned)ceil_div(count, 8), 256, 0, s>>>(count, f); });
+    }
+    int map(int64_t count, const blk::ChunkSum &f, const char *name) {
+        return launch(count, name, [&] { chunk_sum_kernel<<<(unsigned)count, 32, 0, s>>>(f); });
+    }
+    int map(int64_t count, const blk::Transpose &f, const char *name) {
+        const int64_t tr = (f.rows + 31) / 32, tcn = (f.cols + 31) / 32;
+        if (tr * tcn > 0x7FFFFFFFll) return map<blk::Transpose>(count, f, name);
+        return launch(count, name, [&] { transpose_kernel<<<(unsigned)(tr * tcn), 256, 0, s>>>(f, tcn); });
     }
 
     // The attention passes run as tiled kernels (attention.cu) unless the
@@ -79,6 +192,24 @@ struct DevExec {
 
     int gemm(const blk::Gemm &g, const char *name) {
         if (st != REALQ_OK) return 1;
+        if (x6_ok(g)) {
+            const int64_t ldk = (g.K + 7) / 8 * 8;
+            __nv_bfloat16 *Ap = reinterpret_cast<__nv_bfloat16 *>(planes);
+            __nv_bfloat16 *Bp = reinterpret_cast<__nv_bfloat16 *>(planes + 2 * cap);
+            // A: its rows, or the columns of the K x M matrix; B (K x N): its columns
+            X6Split a{g.A, g.lda, g.a_kmajor ? g.K : g.M, g.a_kmajor ? g.M : g.K, g.a_kmajor, Ap, ldk, g.M * ldk};
+            X6Split b{g.B, g.ldb, g.K, g.N, 1, Bp, ldk, g.N * ldk};
+            st = split3(s, a, &b);
+            X6Epi e{};
+            e.mode = X6_STORE;
+            e.C = g.C; e.ldc = g.ldc;
+            e.alpha = g.alpha;
+            e.R = g.R; e.ldr = g.ldr;
+            if (st == REALQ_OK)
+                st = gemm_x6(s, X6Planes{Ap, g.M, g.K, ldk, g.M * ldk}, X6Planes{Bp, g.N, g.K, ldk, g.N * ldk}, g.M, g.N,
+                             g.K, 0, 0, 0, 0, e, err, name);
+            return st != REALQ_OK;
+        }
         if (tc_ok(g)) {
             float *Ah = planes, *Al = planes + cap, *Bh = planes + 2 * cap, *Bl = planes + 3 * cap;
             // A (M x K): rows of A, or A stored K x M (column i of the stored matrix)
@@ -222,7 +353,8 @@ int g_block_tc = 0;   // realq_set_block_products
 char *exec_at(DevExec *X, void *ws, const blk::Dims &dm, int64_t vocab) {
     char *p = static_cast<char *>(ws);
     X->cap = tc_cap(dm, vocab);
-    X->planes = g_block_tc ? reinterpret_cast<float *>(p + kAlign) : nullptr;
+    X->planes = reinterpret_cast<float *>(p + kAlign);
+    X->tf32 = g_block_tc == 1;
     if (g_status_override) {
         X->err = g_status_override;
     } else {

@@ -316,9 +316,7 @@ CUresult encode_tmap_2d_f32(CUtensorMap *map, const void *base, uint64_t inner, 
                           box_outer, swizzle128);
 }
 
-static CUresult encode_tmap_2d(CUtensorMapDataType dt, CUtensorMap *map, const void *base, uint64_t inner,
-                               uint64_t outer, uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_outer,
-                               int swizzle128) {
+static bool load_encode() {
     std::call_once(g_encode_once, [] {
         void *fn = nullptr;
         cudaDriverEntryPointQueryResult q;
@@ -327,7 +325,13 @@ static CUresult encode_tmap_2d(CUtensorMapDataType dt, CUtensorMap *map, const v
             q == cudaDriverEntryPointSuccess)
             g_encode = reinterpret_cast<EncodeFn>(fn);
     });
-    if (!g_encode) return CUDA_ERROR_NOT_FOUND;
+    return g_encode != nullptr;
+}
+
+static CUresult encode_tmap_2d(CUtensorMapDataType dt, CUtensorMap *map, const void *base, uint64_t inner,
+                               uint64_t outer, uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_outer,
+                               int swizzle128) {
+    if (!load_encode()) return CUDA_ERROR_NOT_FOUND;
     cuuint64_t dims[2] = {inner, outer};
     cuuint64_t strides[1] = {row_stride_bytes};
     cuuint32_t box[2] = {box_inner, box_outer};
@@ -337,6 +341,19 @@ static CUresult encode_tmap_2d(CUtensorMapDataType dt, CUtensorMap *map, const v
                     swizzle128 == 2 ? CU_TENSOR_MAP_SWIZZLE_64B
                                     : (swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE),
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+}
+
+CUresult encode_tmap_3d_bf16(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer, uint64_t planes,
+                             uint64_t row_stride_bytes, uint64_t plane_stride_bytes, uint32_t box_inner,
+                             uint32_t box_outer, uint32_t box_planes) {
+    if (!load_encode()) return CUDA_ERROR_NOT_FOUND;
+    cuuint64_t dims[3] = {inner, outer, planes};
+    cuuint64_t strides[2] = {row_stride_bytes, plane_stride_bytes};
+    cuuint32_t box[3] = {box_inner, box_outer, box_planes};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims, strides, box, estr,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
 }
 
 CUresult encode_tmap_2d_f16(CUtensorMap *map, const void *base, uint64_t inner, uint64_t outer,

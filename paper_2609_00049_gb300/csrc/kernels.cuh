@@ -135,6 +135,36 @@ realq_status_t tc_gsum_adam(cudaStream_t s, int64_t m, int64_t N, int nz, const 
 template <typename TY>
 realq_status_t tc_split_diff(cudaStream_t s, int64_t count, const float *x, const TY *y, float *hi, float *lo);
 
+// ------------------------------- fp32 products as bf16x6 (gemm_x6.cu) ---
+// Three bf16 planes of a K-major fp32 operand: element (row, k) of plane p at
+// p[plane * p + row * ld + k]; ld and plane multiples of 8, base 16-byte
+// aligned.  k is the extent the loads see: past it they read zeros.
+struct X6Planes {
+    const __nv_bfloat16 *p;
+    int64_t rows, k, ld, plane;
+};
+enum X6Mode {
+    X6_STORE = 0,       // C = alpha acc (+ R)
+};
+struct X6Epi {
+    int mode;
+    float *C; int64_t ldc;
+    float alpha; const float *R; int64_t ldr;   // X6_STORE (R nullable, may be C)
+};
+// One operand to split into planes: src (rows x cols, row stride lds), as its
+// rows (dst[r * ldd + c]) or, with trans, its columns (dst[c * ldd + r]).
+struct X6Split {
+    const float *src; int64_t lds, rows, cols;
+    int trans;
+    __nv_bfloat16 *dst; int64_t ldd, plane;
+};
+// one or two operands in one launch
+realq_status_t split3(cudaStream_t s, const X6Split &a, const X6Split *b = nullptr);
+// C (M x N) from rows a_row0.. of A and b_row0.. of B, K terms from a_k0 / b_k0 (multiples of 8) on
+realq_status_t gemm_x6(cudaStream_t s, const X6Planes &A, const X6Planes &B, int64_t M, int64_t N, int64_t K,
+                       int64_t a_row0, int64_t b_row0, int64_t a_k0, int64_t b_k0, const X6Epi &e, int *err,
+                       const char *name);
+
 // ------------------------------------------------- activation quantizer ---
 realq_status_t act_quant(cudaStream_t s, int64_t T, int64_t n, const void *X, realq_dtype_t dt, int bits, float a_clip,
                          void *Xq, uint8_t *codes, float *scale);
