@@ -24,9 +24,6 @@
 //             moments and the displacement, and writing the step's hi / lo
 //             planes for the next M update
 //   TC_ACCUM  M += acc (the running product of one row group)
-//   TC_SYRK   M[i][j] -= acc for j >= i only (a symmetric rank-K update of
-//             the upper triangle of M; tiles wholly below the diagonal exit
-//             at once)
 //   TC_BGD_PG the gradient factor of a row group whose OBS used its own
 //             H̄_g:  p = M + lambda_g (A_disp - (W - W0)) - acc (+ W0 Dbar),
 //             acc = ΔW (H̄_g - H̄); written like TC_BGD_P
@@ -189,21 +186,6 @@ __device__ __forceinline__ void accum_rows4(const TcEpi &e, int64_t gi0, int64_t
     }
 }
 
-// TC_SYRK for 4 rows x 4 columns: M -= acc on and above the diagonal
-__device__ __forceinline__ void syrk_rows4(const TcEpi &e, int64_t gi0, int64_t gj, const float *t, int tp) {
-    float4 mp[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) mp[u] = ld4(e.M + (gi0 + u) * e.ldw + gj);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const float *tr = t + u * tp;
-        const int64_t gi = gi0 + u;
-        st4(e.M + gi * e.ldw + gj,
-            make_float4(gj + 0 >= gi ? mp[u].x - tr[0] : mp[u].x, gj + 1 >= gi ? mp[u].y - tr[1] : mp[u].y,
-                        gj + 2 >= gi ? mp[u].z - tr[2] : mp[u].z, gj + 3 >= gi ? mp[u].w - tr[3] : mp[u].w));
-    }
-}
-
 __device__ __forceinline__ float adam_step(const TcEpi &e, float g, float &m, float &v) {
     if (e.sgd) return e.lr * g;
     m = e.b1 * m + (1.f - e.b1) * g;
@@ -259,10 +241,6 @@ __device__ __forceinline__ void epi_apply(const TcEpi &e, int64_t i, int64_t j, 
     }
     if (e.mode == TC_ACCUM) {
         e.M[i * e.ldw + e.col0 + j] += v;
-        return;
-    }
-    if (e.mode == TC_SYRK) {
-        if (j >= i) e.M[i * e.ldw + j] -= v;
         return;
     }
     const int64_t col = e.col0 + j;
@@ -325,16 +303,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         tj = (pid % per) / gm;
     }
     const int64_t i0 = ti * TB, j0 = tj * TN;
-    // a symmetric update touches the upper triangle only: a tile wholly
-    // below the diagonal has nothing to do (uniform over the CTA, before any
-    // barrier or allocation)
-    if (MODE == TC_SYRK && j0 + TN <= i0) return;
     // K split over blockIdx.z: this CTA takes K range [kz0, kz0 + Kz)
     const int64_t kz0 = kchunk > 0 ? (int64_t)blockIdx.z * kchunk : 0;
-    int64_t Kz = kchunk > 0 ? ((K - kz0) < kchunk ? (K - kz0) : kchunk) : K;
-    // a triangular B (zero beyond the output column): this tile's K range
-    // ends at its last column (the wrapper takes no K split with it)
-    if (e.b_tri && Kz > j0 + TN) Kz = j0 + TN;
+    const int64_t Kz = kchunk > 0 ? ((K - kz0) < kchunk ? (K - kz0) : kchunk) : K;
     const int nk = (int)((Kz + KS - 1) / KS);
 
     if (threadIdx.x == 0) {
@@ -473,7 +444,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (MODE == TC_ADAM) adam_rows4(e, i0 + rb, M, gj, T + rb * TP + cc, TP);
                     else if (MODE == TC_BGD_P) bgd_p_rows4(e, i0 + rb, M, gj, T + rb * TP + cc, TP);
                     else if (MODE == TC_BGD_PG) bgd_pg_rows4(e, i0 + rb, gj, T + rb * TP + cc, TP);
-                    else if (MODE == TC_SYRK) syrk_rows4(e, i0 + rb, gj, T + rb * TP + cc, TP);
                     else accum_rows4(e, i0 + rb, gj, T + rb * TP + cc, TP);
                 } else {
                     for (int u = 0; u < 4; ++u) {
@@ -1160,13 +1130,11 @@ realq_status_t launch_x3(cudaStream_t s, const Maps &m, int64_t M, int64_t N, in
         REALQ_TRY(set_smem_limit(reinterpret_cast<const void *>(gemm_x3_kernel<TC_ADAM, TN, false>), SM));
         REALQ_TRY(set_smem_limit(reinterpret_cast<const void *>(gemm_x3_kernel<TC_ACCUM, TN, false>), SM));
         REALQ_TRY(set_smem_limit(reinterpret_cast<const void *>(gemm_x3_kernel<TC_BGD_PG, TN, false>), SM));
-        REALQ_TRY(set_smem_limit(reinterpret_cast<const void *>(gemm_x3_kernel<TC_SYRK, TN, false>), SM));
         switch (e.mode) {
             case TC_STORE: launch_mode<TC_STORE, TN, false>(s, m, grid, M, N, K, k_off, b_row0, e, err, a_row0, kchunk, exact); break;
             case TC_BGD_P: launch_mode<TC_BGD_P, TN, false>(s, m, grid, M, N, K, k_off, b_row0, e, err, a_row0, kchunk, exact); break;
             case TC_ADAM: launch_mode<TC_ADAM, TN, false>(s, m, grid, M, N, K, k_off, b_row0, e, err, a_row0, kchunk, exact); break;
             case TC_ACCUM: launch_mode<TC_ACCUM, TN, false>(s, m, grid, M, N, K, k_off, b_row0, e, err, a_row0, kchunk, exact); break;
-            case TC_SYRK: launch_mode<TC_SYRK, TN, false>(s, m, grid, M, N, K, k_off, b_row0, e, err, a_row0, kchunk, exact); break;
             default: launch_mode<TC_BGD_PG, TN, false>(s, m, grid, M, N, K, k_off, b_row0, e, err, a_row0, kchunk, exact); break;
         }
         return REALQ_OK;
@@ -1240,13 +1208,10 @@ realq_status_t tc_gemm_x3(cudaStream_t s, const TcMaps &maps, int64_t M, int64_t
     const int ks = f16 ? Tile<128, true>::KS : Tile<128>::KS;
     if (kchunk < 0 || (kchunk % ks) != 0 || (kchunk > 0 && e.mode != TC_STORE))
         return fail(REALQ_ERR_INVALID_ARG, "%s: a K split takes a multiple of %d and the store epilogue", name, ks);
-    if (f16 && (e.b_tri || (e.mode != TC_STORE && e.mode != TC_BGD_P && e.mode != TC_ADAM) || !e.ainv || !e.binv))
+    if (f16 && ((e.mode != TC_STORE && e.mode != TC_BGD_P && e.mode != TC_ADAM) || !e.ainv || !e.binv))
         return fail(REALQ_ERR_INVALID_ARG, "%s: f16x3 takes the store, gradient-factor or Adam epilogue with row "
                     "scales", name);
-    if (e.mode < TC_STORE || e.mode > TC_SYRK) return fail(REALQ_ERR_INVALID_ARG, "%s: bad epilogue mode", name);
-    if (e.mode == TC_SYRK && (a_row0 != 0 || b_row0 != 0 || M != N))
-        return fail(REALQ_ERR_INVALID_ARG, "%s: a symmetric update takes a square product from row 0", name);
-    if (e.b_tri && kchunk > 0) return fail(REALQ_ERR_INVALID_ARG, "%s: a triangular B takes no K split", name);
+    if (e.mode < TC_STORE || e.mode > TC_BGD_PG) return fail(REALQ_ERR_INVALID_ARG, "%s: bad epilogue mode", name);
     if (e.affine && (kchunk > 0 || e.mode != TC_STORE))
         return fail(REALQ_ERR_INVALID_ARG, "%s: the affine store takes no K split", name);
     const MapPair &mp = *reinterpret_cast<const MapPair *>(maps.storage);

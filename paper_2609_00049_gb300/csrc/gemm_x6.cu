@@ -86,7 +86,14 @@ __global__ void __launch_bounds__(THREADS, 1)
         i0 = (first + (pid % per) % gm) * TM;
         j0 = ((pid % per) / gm) * TN;
     }
-    const int64_t kbeg = 0, kend = K;
+    if (e.mode == X6_UPPER && e.joff + j0 + TN <= i0) return;   // wholly below the diagonal (uniform over the CTA)
+    // triangular operands shorten the K range: a_lo A(i, k) = 0 for k < i,
+    // b_lo B(j, k) = 0 for k < j, b_hi B(j, k) = 0 for k > j
+    int64_t kbeg = 0, kend = K;
+    if (e.a_lo && i0 > kbeg) kbeg = i0;
+    if (e.b_lo && j0 > kbeg) kbeg = j0;
+    kbeg = kbeg / KS * KS;
+    if (e.b_hi && kend > j0 + TN) kend = j0 + TN;
     const int nk = kend > kbeg ? (int)((kend - kbeg + KS - 1) / KS) : 0;
 
     if (threadIdx.x == 0) {
@@ -184,6 +191,17 @@ __global__ void __launch_bounds__(THREADS, 1)
         // ------- drain warps: TMEM slice -> fp32 registers (lane quarter, column half) -------
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t col_base = (uint32_t)((warp >> 2) * (TN / 2));
+        if (e.mode != X6_STORE || e.R) {
+            // the tile that the epilogue combines with, into L2 while the MMAs
+            // run: one 128-byte line per thread and step
+            const float *src = e.mode == X6_STORE ? e.R : e.C;
+            const int64_t lds = e.mode == X6_STORE ? e.ldr : e.ldc;
+            const int64_t jm = N < j0 + TN ? N : j0 + TN;
+            for (int l = threadIdx.x; l < TM * (TN / 32); l += DRAIN_WARPS * 32) {
+                const int64_t gi = i0 + l / (TN / 32), gj = j0 + (l % (TN / 32)) * 32;
+                if (gi < M && gj < jm) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + gi * lds + gj));
+            }
+        }
         for (int it = 0; it < nk; ++it) {
             const int b = it & 1;
             const bool ok = tc::mbar_wait(tc::smem_u32(&accf[b]), (uint32_t)(it >> 1) & 1u, abort_flag);
@@ -217,17 +235,30 @@ __global__ void __launch_bounds__(THREADS, 1)
 #pragma unroll
         for (int c0 = 0; c0 < TN / 2; c0 += 32) {
             const int64_t gj = j0 + (warp >> 2) * (TN / 2) + c0 + lane;
+            // rows 0 .. top - 1 of the block are written; what C is combined
+            // with is read first, 16 rows at a time (a load after a store to C
+            // would wait for it)
+            const int rows = (int)(M - gi0 < 32 ? (M - gi0 > 0 ? M - gi0 : 0) : 32);
+            const bool upper = e.mode == X6_UPPER;
+            const bool fold = upper || (e.mode == X6_ADD && gj >= e.nstore) || (e.mode == X6_STORE && e.R);
+            const float *src = (e.mode == X6_STORE ? e.R : e.C) + gi0 * (e.mode == X6_STORE ? e.ldr : e.ldc) + gj;
+            const int64_t lds = e.mode == X6_STORE ? e.ldr : e.ldc;
+            int top = upper && gj + e.joff - gi0 + 1 < rows ? (int)(gj + e.joff - gi0 + 1) : rows;
+            if (gj >= N) top = 0;
 #pragma unroll
             for (int q = 0; q < 32; ++q) st[lane * STG_PITCH + q] = acc[c0 + q];
             __syncwarp();
-            if (gj < N) {
-                const int rows = (int)(M - gi0 < 32 ? (M - gi0 > 0 ? M - gi0 : 0) : 32);
-#pragma unroll 8
-                for (int r = 0; r < rows; ++r) {
-                    float v = e.alpha * st[r * STG_PITCH + lane];
-                    if (e.R) v += e.R[(gi0 + r) * e.ldr + gj];
-                    e.C[(gi0 + r) * e.ldc + gj] = v;
-                }
+            float *dst = e.C + gi0 * e.ldc + gj;
+#pragma unroll 1
+            for (int r0 = 0; r0 < top; r0 += 16) {
+                float old[16];
+#pragma unroll
+                for (int u = 0; u < 16; ++u) old[u] = fold && r0 + u < top ? src[u * lds] : 0.f;
+#pragma unroll
+                for (int u = 0; u < 16; ++u)
+                    if (r0 + u < top) dst[u * e.ldc] = old[u] + e.alpha * st[(r0 + u) * STG_PITCH + lane];
+                src += 16 * lds;
+                dst += 16 * e.ldc;
             }
             __syncwarp();
         }

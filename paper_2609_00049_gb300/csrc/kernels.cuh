@@ -51,7 +51,7 @@ struct GemmArgs {
 realq_status_t gemm_f32(cudaStream_t s, AMode am, EpiMode em, const GemmArgs &g, const char *name);
 
 // ------------------------------------------- tensor-core tf32x3 GEMM ---
-enum TcMode { TC_STORE = 0, TC_BGD_P = 1, TC_ADAM = 2, TC_ACCUM = 3, TC_BGD_PG = 4, TC_SYRK = 5 };
+enum TcMode { TC_STORE = 0, TC_BGD_P = 1, TC_ADAM = 2, TC_ACCUM = 3, TC_BGD_PG = 4 };
 struct TcEpi {
     int mode;
     float *C; int64_t ldc;                                   // TC_STORE
@@ -62,7 +62,6 @@ struct TcEpi {
     float *Wm; float *mA; float *vA; float *D; float *Sh; float *Sl;  // TC_ADAM (ldw, col0 shared)
     float lr, b1, b2, eps, bc1, bc2; int sgd;
     int64_t czs;                                             // TC_STORE with a K split: C of split z at C + z czs
-    int b_tri;   // B(j, k) = 0 for k > j (K range relative to the output column): a CTA's K ends at its last column
     // TC_STORE without a K split: C = alpha_s acc + R (R nullable, row stride ldr) when affine is set
     int affine; float alpha_s; const float *R; int64_t ldr;
     // f16x3 maps: the accumulator is in units of the operands' power-of-two
@@ -145,11 +144,15 @@ struct X6Planes {
 };
 enum X6Mode {
     X6_STORE = 0,       // C = alpha acc (+ R)
+    X6_UPPER = 1,   // C[i][j] += alpha acc for j + joff >= i (tiles wholly below are skipped)
+    X6_ADD = 2,         // C = alpha acc for columns < nstore, C += alpha acc for the others
 };
 struct X6Epi {
     int mode;
     float *C; int64_t ldc;
-    float alpha; const float *R; int64_t ldr;   // X6_STORE (R nullable, may be C)
+    float alpha; const float *R; int64_t ldr;   // R: X6_STORE (nullable, may be C)
+    int64_t joff, nstore;
+    int a_lo, b_lo, b_hi;                       // A(i, k) = 0 for k < i, B(j, k) = 0 for k < j, B(j, k) = 0 for k > j
 };
 // One operand to split into planes: src (rows x cols, row stride lds), as its
 // rows (dst[r * ldd + c]) or, with trans, its columns (dst[c * ldd + r]).
@@ -196,6 +199,11 @@ realq_status_t hessian_cross_tc(cudaStream_t s, int64_t n, int64_t T, const void
 int hessian_splits_tiles(int64_t tiles, int64_t T, int sms);
 
 // --------------------------------------------------------------- prepare ---
+// A diagonal block of n <= kCholBlock columns at A (row stride ld, upper
+// triangle, zeros below): U = R^-1 of its reverse-order Cholesky factor, in
+// place; the first bad pivot's column (col0 + its index) into *status.
+constexpr int64_t kCholBlock = 512;
+realq_status_t chol_inv_block(cudaStream_t s, int64_t ld, float *A, int64_t n, int64_t col0, int *status);
 size_t prepare_ws_bytes(int64_t n);
 realq_status_t prepare(cudaStream_t s, int64_t n, double norm, float damp, const float *H, float *U, float *Hbar,
                        uint8_t *dead, int64_t *fail_col, void *ws, size_t ws_bytes);

@@ -7,12 +7,16 @@
 // the inverse Hessian after the Schur-complement downdates of columns < j,
 // which is what the OBS step of Eq. (gptq_update) consumes.
 //
-// Both factorizations are blocked with 64-wide blocks: a one-CTA kernel
-// factors / inverts the diagonal block in shared memory, the off-diagonal work
-// runs as fp32 GEMMs.  A pivot that is not positive (or not finite) records its
-// column in the workspace status word; prepare reads it once at the end, the
-// deferred variant leaves it for realq_prepare_status (a captured step reads
-// no host memory).
+// Up to 512 columns one thread-block cluster does the whole factor
+// (chol_cluster.cu).  Wider inputs are blocked by 512: the cluster factors and
+// inverts each diagonal block, and everything beside it is a product of depth
+// 512 with fp32 accuracy on the tensor cores (gemm_x6.cu), spread over three
+// streams (prepare_blocked below).  The allocation-free entry point, whose
+// scratch has no room for operand planes, keeps 64-wide steps on the CUDA
+// cores (prepare_steps).  A pivot that is not positive (or not finite) records
+// its column in the workspace status word; prepare reads it once at the end,
+// the deferred variant leaves it for realq_prepare_status (a captured step
+// reads no host memory).
 #include "kernels.cuh"
 
 #include <vector>
@@ -261,25 +265,20 @@ __global__ void scale_kernel(int64_t count, float div, const float *in, float *o
 }
 
 constexpr size_t align256(size_t x) { return (x + 255) / 256 * 256; }
-constexpr int KSPLIT_MAX = 16;   // K slices of the triangular-inverse panel product
-constexpr size_t prepare_bytes_split(int64_t n, int slices) {
+constexpr size_t prepare_bytes(int64_t n) {
     return align256(sizeof(int)) + align256(sizeof(float)) + align256((size_t)NB * NB * sizeof(float)) +
-           align256((size_t)slices * n * NB * sizeof(float));
+           align256((size_t)n * NB * sizeof(float));
 }
-constexpr size_t prepare_bytes(int64_t n) { return prepare_bytes_split(n, 1); }
-// tf32 hi / lo planes of two panels (n x NB each), for the rank-NB updates on
-// the tensor cores (two sets: a step's panel is split while the previous
-// step's update may still read the other set)
-constexpr size_t tc_panel_bytes(int64_t n) { return 4 * align256((size_t)n * NB * sizeof(float)); }
-// the triangular inverse's product on the tensor cores: planes of U^T (n x n,
-// filled block column by block column as U's row blocks become final) and of
-// the row block R[K, K+1:] (NB x n, at its global columns)
-constexpr size_t tc_trtri_bytes(int64_t n) {
-    return 2 * align256((size_t)n * n * sizeof(float)) + 2 * align256((size_t)NB * n * sizeof(float));
+// Operand planes of the blocked preparation (three bf16 planes each, 512
+// terms deep): U_KK, the panel A[0:k0, K] before its solve, kPanels panels
+// R[0:k0, K] (a step's updates may still read the earlier ones), the row block
+// of U before its product with U_KK, and its transpose after it.
+constexpr int64_t PB = kCholBlock;
+constexpr int kPanels = 3;
+constexpr size_t planes_bytes(int64_t rows) { return align256((size_t)rows * PB * 3 * sizeof(__nv_bfloat16)); }
+constexpr size_t blocked_bytes(int64_t n) {
+    return n <= PB ? 0 : planes_bytes(PB) + (size_t)(1 + kPanels + 2) * planes_bytes(n);
 }
-// the rank-NB update above the diagonal takes the tensor cores from this many
-// rows on (below it the fp32 tiles, whose work is small)
-constexpr int64_t kTcUpdateRows = 512;
 
 // Scratch of the allocation-free entry point, sized for n <= REALQ_PREPARE_NOALLOC_MAX_N.
 // Every GPU that loads the library holds it until the process exits.
@@ -301,9 +300,7 @@ realq_status_t noalloc_scratch(void **out) {
 
 }  // namespace
 
-size_t prepare_ws_bytes(int64_t n) {
-    return prepare_bytes_split(n, KSPLIT_MAX) + tc_panel_bytes(n) + tc_trtri_bytes(n);
-}
+size_t prepare_ws_bytes(int64_t n) { return prepare_bytes(n) + blocked_bytes(n); }
 
 realq_status_t prepare_impl(cudaStream_t s, int64_t n, double norm, float damp, const float *H, float *U, float *Hbar,
                             uint8_t *dead, int64_t *fail_col, void *ws, size_t ws_bytes, bool overlap, bool sync);
@@ -325,10 +322,10 @@ realq_status_t prepare_noalloc(cudaStream_t s, int64_t n, int64_t T, float damp,
 struct AuxStream {
     int device = -1, priority = 0;
     cudaStream_t caller = nullptr;
-    cudaStream_t stream = nullptr;       // U row work
+    cudaStream_t stream = nullptr;       // the rows of U
     cudaStream_t wide = nullptr;         // the look-ahead's wide trailing updates
     cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
-    std::vector<cudaEvent_t> steps, pdone, wdone;
+    std::vector<cudaEvent_t> steps, pdone, wdone, rdone;
 };
 static thread_local std::vector<AuxStream> g_aux;
 
@@ -351,7 +348,7 @@ realq_status_t aux_for(cudaStream_t s, int64_t nsteps, AuxStream **out) {
         found = &g_aux.back();
     }
     AuxStream &a = *found;
-    for (std::vector<cudaEvent_t> *v : {&a.steps, &a.pdone, &a.wdone}) {
+    for (std::vector<cudaEvent_t> *v : {&a.steps, &a.pdone, &a.wdone, &a.rdone}) {
         while ((int64_t)v->size() < nsteps) {
             cudaEvent_t e;
             REALQ_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
@@ -372,6 +369,177 @@ realq_status_t prepare_deferred(cudaStream_t s, int64_t n, double norm, float da
     return prepare_impl(s, n, norm, damp, H, U, Hbar, dead, nullptr, ws, ws_bytes, !profiling(), false);
 }
 
+// Inputs of up to n = 64 nbk columns in 64-wide steps on the CUDA cores, one
+// stream: for each step the diagonal factor (and inverse), the panel, the
+// rank-64 update of what lies above, and row block K of U:
+//   U[K, K] = R_KK^-1,  U[K, K+1:] = -U[K, K] (R[K, K+1:] U[K+1:, K+1:])
+// (after step K no later step reads row block K of R).
+static realq_status_t prepare_steps(cudaStream_t s, int64_t n, float *U, float *Vd, float *panel, int *status) {
+    const int64_t plane = n * NB;
+    const int nbk = ceil_div(n, NB);
+    for (int K = nbk - 1; K >= 0; --K) {
+        const int64_t k0 = (int64_t)K * NB;
+        const int kb = (int)std::min<int64_t>(NB, n - k0);
+        const int64_t k1 = k0 + kb;
+        {
+            Launch L("chol_diag", s);
+            chol_diag_kernel<<<1, 128, 0, s>>>(n, U, k0, kb, status, Vd);
+        }
+        REALQ_TRY(check_launch("chol_diag"));
+        if (k0 > 0) {
+            // rows above the block: R[0:k0, K] = A[0:k0, K] R_KK^-T (in place; one
+            // column tile, so every CTA reads only the rows it writes)
+            GemmArgs pg{};
+            pg.M = k0; pg.N = kb; pg.K = kb;
+            pg.A = U + k0; pg.lda = n;
+            pg.B = Vd; pg.ldb = NB;
+            pg.C = U + k0; pg.ldc = n;
+            pg.alpha = 1.f;
+            REALQ_TRY(gemm_f32(s, A_ROW, EPI_STORE, pg, "chol_panel"));
+            const int64_t nt0 = k0 / NB;
+            {
+                Launch L("chol_update", s);
+                chol_update_kernel<<<(unsigned)(nt0 * (nt0 + 1) / 2), 256, 0, s>>>(n, U, k0, kb, 0);
+            }
+            REALQ_TRY(check_launch("chol_update"));
+        }
+        if (k1 < n) {
+            const int64_t r = n - k1;
+            // X = R[K, K+1:] U[K+1:, K+1:] (U upper: a column tile's K range ends
+            // at its last column)
+            GemmArgs g{};
+            g.M = kb; g.N = r; g.K = r;
+            g.A = U + k0 * n + k1; g.lda = n;
+            g.B = U + k1 * n + k1; g.ldb = n;
+            g.C = panel; g.ldc = n;
+            g.cplane = plane; g.b_upper = 1;
+            g.alpha = 1.f;
+            REALQ_TRY(gemm_f32(s, A_ROW, EPI_STORE, g, "trtri_trmm"));
+            // U[K, K+1:] = -U_KK X, U_KK read from A[K, K] (upper, zeros below)
+            GemmArgs h{};
+            h.M = kb; h.N = r; h.K = kb;
+            h.A = U + k0 * n + k0; h.lda = n;
+            h.B = panel; h.ldb = n; h.nsum_b = 1; h.bplane = plane;
+            h.C = U + k0 * n + k1; h.ldc = n;
+            h.alpha = -1.f;
+            REALQ_TRY(gemm_f32(s, A_ROW, EPI_STORE, h, "trtri_panel"));
+        }
+    }
+    return REALQ_OK;
+}
+
+// Wider inputs, 512 columns at a time.  Step K (block K = columns k0 .. k1):
+//   s      the cluster factors and inverts A[K, K] (in place: U_KK); the panel
+//          R[0:k0, K] = A[0:k0, K] U_KK^T; the update of the next block's
+//          columns, A[0:k0, K-1] -= R[0:k0, K] R[K-1, K]^T (upper)
+//   wide   the update of the columns before those, overlapped with the next
+//          diagonal block and panel (look-ahead)
+//   rows   row block K of U.  S[I, j] = sum over K of R[I, K] U[K, j] is
+//          accumulated in place of R[I, j] (which step j consumed as planes):
+//            U[K, K+1:] = -U_KK S[K, K+1:], then for the rows I above
+//            S[I, K] = R[I, K] U_KK and S[I, K+1:] += R[I, K] U[K, K+1:].
+// So every product has depth 512 and as many tiles as the matrix gives it,
+// where one product per row block of U with a depth of up to n had few tiles
+// and a long chain.  A product's operands are three bf16 planes each.
+static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *status, int *status_tc,
+                                      unsigned char *planes, bool overlap) {
+    Carve cv(planes);
+    auto take = [&](int64_t rows) { return cv.take<__nv_bfloat16>((size_t)rows * PB * 3); };
+    __nv_bfloat16 *Vp = take(PB), *Ap = take(n), *Rp[kPanels], *Sp, *Up;
+    for (int i = 0; i < kPanels; ++i) Rp[i] = take(n);
+    Sp = take(n);
+    Up = take(n);
+    const int nbk = ceil_div(n, PB);
+    AuxStream *aux = nullptr;
+    if (overlap) REALQ_TRY(aux_for(s, nbk, &aux));
+    cudaStream_t rs = aux ? aux->stream : s, wd = aux ? aux->wide : s;
+    if (aux) {
+        // the side streams follow everything already on s
+        REALQ_CUDA_TRY(cudaEventRecord(aux->ev[0], s));
+        REALQ_CUDA_TRY(cudaStreamWaitEvent(rs, aux->ev[0], 0));
+        REALQ_CUDA_TRY(cudaStreamWaitEvent(wd, aux->ev[0], 0));
+    }
+    // planes of rows x PB terms, k terms of which exist
+    auto op = [&](const __nv_bfloat16 *p, int64_t rows, int64_t k) { return X6Planes{p, rows, k, PB, rows * PB}; };
+    for (int K = nbk - 1; K >= 0; --K) {
+        const int64_t k0 = (int64_t)K * PB, kb = std::min<int64_t>(PB, n - k0), k1 = k0 + kb, r = n - k1;
+        __nv_bfloat16 *Rk = Rp[K % kPanels];
+        REALQ_TRY(chol_inv_block(s, n, U + k0 * n + k0, kb, k0, status));
+        if (k0 > 0) {
+            // the planes of U_KK and of the panel, and the panel's solve (U_KK upper: terms k >= j)
+            const X6Split sv{U + k0 * n + k0, n, kb, kb, 0, Vp, PB, kb * PB}, sa{U + k0, n, k0, kb, 0, Ap, PB, k0 * PB};
+            REALQ_TRY(split3(s, sa, &sv));
+            X6Epi e{};
+            e.mode = X6_STORE;
+            e.C = U + k0; e.ldc = n;
+            e.alpha = 1.f;
+            e.b_lo = 1;
+            REALQ_TRY(gemm_x6(s, op(Ap, k0, kb), op(Vp, kb, kb), k0, kb, kb, 0, 0, 0, 0, e, status_tc, "chol_panel_tc"));
+            // (the planes that step K + kPanels left here are no longer read)
+            if (aux && K + kPanels < nbk) REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->rdone[K + kPanels], 0));
+            const X6Split sr{U + k0, n, k0, kb, 0, Rk, PB, k0 * PB};
+            REALQ_TRY(split3(s, sr));
+            if (aux) {
+                REALQ_CUDA_TRY(cudaEventRecord(aux->pdone[K], s));
+                REALQ_CUDA_TRY(cudaStreamWaitEvent(rs, aux->pdone[K], 0));
+            }
+            const int64_t kw = k0 - PB;   // rows and columns of the wide part
+            if (aux) REALQ_CUDA_TRY(cudaStreamWaitEvent(wd, aux->pdone[K], 0));
+            // the narrow part's columns were last written by the wide part of step K + 1
+            if (aux && K + 1 < nbk) REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->wdone[K + 1], 0));
+            X6Epi u{};
+            u.mode = X6_UPPER;
+            u.alpha = -1.f;
+            u.C = U + kw; u.ldc = n;
+            u.joff = kw;
+            REALQ_TRY(gemm_x6(s, op(Rk, k0, kb), op(Rk, k0, kb), k0, PB, kb, 0, kw, 0, 0, u, status_tc,
+                              "chol_update_tc"));
+            if (kw > 0) {
+                X6Epi w{};
+                w.mode = X6_UPPER;
+                w.alpha = -1.f;
+                w.C = U; w.ldc = n;
+                REALQ_TRY(gemm_x6(wd, op(Rk, k0, kb), op(Rk, k0, kb), kw, kw, kb, 0, 0, 0, 0, w, status_tc,
+                                  "chol_update_tc"));
+            }
+            if (aux) REALQ_CUDA_TRY(cudaEventRecord(aux->wdone[K], wd));
+        } else if (aux) {
+            REALQ_CUDA_TRY(cudaEventRecord(aux->steps[K], s));
+            REALQ_CUDA_TRY(cudaStreamWaitEvent(rs, aux->steps[K], 0));
+        }
+        if (r > 0) {
+            // U[K, K+1:] = -U_KK S[K, K+1:] (U_KK upper: terms k >= i)
+            const X6Split ss{U + k0 * n + k1, n, kb, r, 1, Sp, PB, r * PB}, sv{U + k0 * n + k0, n, kb, kb, 0, Up, PB, kb * PB};
+            REALQ_TRY(split3(rs, ss, &sv));
+            X6Epi e{};
+            e.mode = X6_STORE;
+            e.C = U + k0 * n + k1; e.ldc = n;
+            e.alpha = -1.f;
+            e.a_lo = 1;
+            REALQ_TRY(gemm_x6(rs, op(Up, kb, kb), op(Sp, r, kb), kb, r, kb, 0, 0, 0, 0, e, status_tc, "trtri_panel_tc"));
+        }
+        if (k0 > 0) {
+            const int64_t rr = n - k0;
+            const X6Split su{U + k0 * n + k0, n, kb, rr, 1, Up, PB, rr * PB};
+            REALQ_TRY(split3(rs, su));
+            X6Epi e{};
+            e.mode = X6_ADD;
+            e.alpha = 1.f;
+            e.C = U + k0; e.ldc = n;
+            e.nstore = kb;
+            REALQ_TRY(gemm_x6(rs, op(Rk, k0, kb), op(Up, rr, kb), k0, rr, kb, 0, 0, 0, 0, e, status_tc, "trtri_update_tc"));
+            if (aux) REALQ_CUDA_TRY(cudaEventRecord(aux->rdone[K], rs));
+        }
+    }
+    if (aux) {
+        REALQ_CUDA_TRY(cudaEventRecord(aux->ev[1], rs));
+        REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->ev[1], 0));
+        REALQ_CUDA_TRY(cudaEventRecord(aux->ev[2], wd));
+        REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->ev[2], 0));
+    }
+    return REALQ_OK;
+}
+
 realq_status_t prepare_impl(cudaStream_t s, int64_t n, double norm, float damp, const float *H, float *U, float *Hbar,
                             uint8_t *dead, int64_t *fail_col, void *ws, size_t ws_bytes, bool overlap, bool sync) {
     Carve cv(ws);
@@ -379,38 +547,8 @@ realq_status_t prepare_impl(cudaStream_t s, int64_t n, double norm, float damp, 
     float *lam = cv.take<float>(1);
     float *Vd = cv.take<float>((size_t)NB * NB);
     float *panel = cv.take<float>(0);
-    // the wide rank-NB updates on the tensor cores when the workspace has
-    // room for the panel planes besides one panel slice (otherwise the fp32
-    // tiles) and n suits the product
-    const bool tc_update = n % 4 == 0 && n > kTcUpdateRows && tc_gemm_eligible(n, n) &&
-                           ws_bytes >= prepare_bytes_split(n, 1) + tc_panel_bytes(n);
-    const bool tc_trtri = tc_update && ws_bytes >= prepare_bytes_split(n, 1) + tc_panel_bytes(n) + tc_trtri_bytes(n);
-    const size_t reserve = (tc_update ? tc_panel_bytes(n) : 0) + (tc_trtri ? tc_trtri_bytes(n) : 0);
-    // as many K slices of the panel product as the workspace holds
-    int slices = 1;
-    while (slices < KSPLIT_MAX && prepare_bytes_split(n, slices + 1) + reserve <= ws_bytes) ++slices;
-    const int64_t plane = n * NB;
-    float *Pp[4] = {nullptr, nullptr, nullptr, nullptr};   // set 0 hi, lo; set 1 hi, lo
-    float *UTh = nullptr, *UTl = nullptr, *Rh = nullptr, *Rl = nullptr;
-    TcMaps pmaps[2], tmaps;
-    if (tc_update) {
-        Carve pc(reinterpret_cast<unsigned char *>(ws) + prepare_bytes_split(n, slices));
-        for (int i = 0; i < 4; ++i) Pp[i] = pc.take<float>((size_t)n * NB);
-        for (int st = 0; st < 2; ++st)
-            REALQ_TRY(tc_make_maps(&pmaps[st], Pp[2 * st], Pp[2 * st + 1], n, NB, NB, Pp[2 * st], Pp[2 * st + 1], n,
-                                   NB, NB));
-        if (tc_trtri) {
-            UTh = pc.take<float>((size_t)n * n);
-            UTl = pc.take<float>((size_t)n * n);
-            Rh = pc.take<float>((size_t)NB * n);
-            Rl = pc.take<float>((size_t)NB * n);
-            // A: the row block R[K, K+1:] (NB rows, columns at their global
-            // index); B: rows of U^T, so that both take K from column k1 on
-            REALQ_TRY(tc_make_maps(&tmaps, Rh, Rl, NB, n, n, UTh, UTl, n, n, n));
-        }
-    }
     // status[0]: the failing column (-1: none); status[1]: timeout bits of
-    // the tensor-core updates (the same 256-byte slot of the workspace)
+    // the tensor-core products (the same 256-byte slot of the workspace)
     int *status_tc = status + 1;
     REALQ_CUDA_TRY(cudaMemsetAsync(status, 0xFF, sizeof(int), s));
     REALQ_CUDA_TRY(cudaMemsetAsync(status_tc, 0, sizeof(int), s));
@@ -425,152 +563,13 @@ realq_status_t prepare_impl(cudaStream_t s, int64_t n, double norm, float damp, 
         prep_damp_kernel<<<1, 1024, 0, s>>>(n, U, damp, lam);
     }
     REALQ_TRY(check_launch("prepare_damp"));
-    // Reverse-order blocked Cholesky Hd = R R^T, with U = R^-1 formed block row
-    // by block row as soon as a row block of R is final: after step K no later
-    // step reads row block K of R, and
-    //   U[K, K] = R_KK^-1,  U[K, K+1:] = -U[K, K] (R[K, K+1:] U[K+1:, K+1:]).
-    const int nbk = ceil_div(n, NB);
-    // Row block K of U touches rows >= k0 only, the later Cholesky steps rows
-    // < k0 only: with overlap, the U row work runs on an auxiliary stream that
-    // starts after the diagonal step of K (which wrote U_KK into A[K, K]).
-    if (tc_trtri) {
-        // U^T's planes are filled on and below the diagonal, block column by
-        // block column; what lies above it is read as zeros
-        REALQ_CUDA_TRY(cudaMemsetAsync(UTh, 0, (size_t)n * n * sizeof(float), s));
-        REALQ_CUDA_TRY(cudaMemsetAsync(UTl, 0, (size_t)n * n * sizeof(float), s));
-    }
-    AuxStream *aux = nullptr;
-    if (overlap && nbk > 1) REALQ_TRY(aux_for(s, nbk, &aux));
-    cudaStream_t rs = aux ? aux->stream : s;
-    if (aux) {
-        REALQ_CUDA_TRY(cudaEventRecord(aux->ev[0], s));
-        REALQ_CUDA_TRY(cudaStreamWaitEvent(rs, aux->ev[0], 0));
-    }
-    std::vector<char> wide_pending(nbk + 1, 0);
-    bool wide_used = false;
-    for (int K = nbk - 1; K >= 0; --K) {
-        const int64_t k0 = (int64_t)K * NB;
-        const int kb = (int)std::min<int64_t>(NB, n - k0);
-        const int64_t k1 = k0 + kb;
-        {
-            Launch L("chol_diag", s);
-            chol_diag_kernel<<<1, 128, 0, s>>>(n, U, k0, kb, status, Vd);
-        }
-        REALQ_TRY(check_launch("chol_diag"));
-        if (aux && (k1 < n || tc_trtri)) {
-            REALQ_CUDA_TRY(cudaEventRecord(aux->steps[K], s));
-            REALQ_CUDA_TRY(cudaStreamWaitEvent(rs, aux->steps[K], 0));
-        }
-        if (k0 > 0) {
-            // rows above the block: R[0:k0, K] = A[0:k0, K] R_KK^-T (in place; one
-            // column tile, so every CTA reads only the rows it writes)
-            GemmArgs pg{};
-            pg.M = k0; pg.N = kb; pg.K = kb;
-            pg.A = U + k0; pg.lda = n;
-            pg.B = Vd; pg.ldb = NB;
-            pg.C = U + k0; pg.ldc = n;
-            pg.alpha = 1.f;
-            REALQ_TRY(gemm_f32(s, A_ROW, EPI_STORE, pg, "chol_panel"));
-            // Rank-kb update of the block above.  Look-ahead: the next step
-            // needs only tile column nt0 - 1 (its diagonal block and its
-            // panel), which is updated at once; the other columns ("wide")
-            // run on a second stream, overlapped with the next diagonal
-            // factorisation and panel, and the next narrow update waits for
-            // them because it touches their last column.
-            const int64_t nt0 = k0 / NB;
-            const int64_t nwide = (nt0 - 1) * nt0 / 2;
-            if (aux && nwide > 0) {
-                REALQ_CUDA_TRY(cudaEventRecord(aux->pdone[K], s));
-                REALQ_CUDA_TRY(cudaStreamWaitEvent(aux->wide, aux->pdone[K], 0));
-            }
-            if (aux && K + 1 < nbk && wide_pending[K + 1]) REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->wdone[K + 1], 0));
-            {
-                Launch L("chol_update", s);
-                chol_update_kernel<<<(unsigned)nt0, 256, 0, s>>>(n, U, k0, kb, nwide);
-            }
-            REALQ_TRY(check_launch("chol_update"));
-            if (nwide > 0) {
-                cudaStream_t ws_ = aux ? aux->wide : s;
-                const int64_t kw = k0 - NB;   // rows and columns of the wide part
-                if (tc_update && kw >= kTcUpdateRows) {
-                    // U[0:kw, 0:kw] (upper) -= P P^T with P = R[0:kw, K], as
-                    // a tf32x3 symmetric product on the tensor cores
-                    const int st = K & 1;
-                    REALQ_TRY(tc_split_rows(ws_, kw, kb, U + k0, n, Pp[2 * st], Pp[2 * st + 1], NB, NB));
-                    TcEpi e{};
-                    e.mode = TC_SYRK;
-                    e.M = U;
-                    e.ldw = n;
-                    REALQ_TRY(tc_gemm_x3(ws_, pmaps[st], kw, kw, NB, 0, 0, e, status_tc, "chol_update_tc"));
-                } else {
-                    Launch L("chol_update", ws_);
-                    chol_update_kernel<<<(unsigned)nwide, 256, 0, ws_>>>(n, U, k0, kb, 0);
-                }
-                REALQ_TRY(check_launch("chol_update"));
-                if (aux) {
-                    REALQ_CUDA_TRY(cudaEventRecord(aux->wdone[K], aux->wide));
-                    wide_pending[K] = 1;
-                    wide_used = true;
-                }
-            }
-        }
-        if (k1 < n && tc_trtri) {
-            const int64_t r = n - k1;
-            // X = R[K, K+1:] U[K+1:, K+1:] on the tensor cores: the planes of
-            // the row block, then X = R_K (U^T)^T with U^T's rows k1.. (a
-            // column tile's K range ends at its last column: U is upper)
-            REALQ_TRY(tc_split_rows(rs, kb, r, U + k0 * n + k1, n, Rh + k1, Rl + k1, n, r));
-            TcEpi e{};
-            e.mode = TC_STORE;
-            e.C = panel;
-            e.ldc = n;
-            e.b_tri = 1;
-            REALQ_TRY(tc_gemm_x3(rs, tmaps, kb, r, r, (int)k1, (int)k1, e, status_tc, "trtri_trmm_tc"));
-            // U[K, K+1:] = -U_KK X, U_KK read from A[K, K] (upper, zeros below)
-            GemmArgs h{};
-            h.M = kb; h.N = r; h.K = kb;
-            h.A = U + k0 * n + k0; h.lda = n;
-            h.B = panel; h.ldb = n; h.nsum_b = 1; h.bplane = plane;
-            h.C = U + k0 * n + k1; h.ldc = n;
-            h.alpha = -1.f;
-            REALQ_TRY(gemm_f32(rs, A_ROW, EPI_STORE, h, "trtri_panel"));
-        } else if (k1 < n) {
-            const int64_t r = n - k1;
-            // X = R[K, K+1:] U[K+1:, K+1:] (U upper: a column tile's K range ends
-            // at its last column), K split into fixed-order slices
-            const int ks = (int)std::max<int64_t>(1, std::min<int64_t>(slices, r / 256));
-            GemmArgs g{};
-            g.M = kb; g.N = r; g.K = r;
-            g.A = U + k0 * n + k1; g.lda = n;
-            g.B = U + k1 * n + k1; g.ldb = n;
-            g.C = panel; g.ldc = n;
-            g.ksplit = ks; g.cplane = plane; g.b_upper = 1;
-            g.alpha = 1.f;
-            REALQ_TRY(gemm_f32(rs, A_ROW, EPI_STORE, g, "trtri_trmm"));
-            // U[K, K+1:] = -U_KK X, U_KK read from A[K, K] (upper, zeros below)
-            GemmArgs h{};
-            h.M = kb; h.N = r; h.K = kb;
-            h.A = U + k0 * n + k0; h.lda = n;
-            h.B = panel; h.ldb = n; h.nsum_b = ks; h.bplane = plane;
-            h.C = U + k0 * n + k1; h.ldc = n;
-            h.alpha = -1.f;
-            REALQ_TRY(gemm_f32(rs, A_ROW, EPI_STORE, h, "trtri_panel"));
-        }
-        // row block K of U is final: its transpose joins U^T's planes for the
-        // later steps' products
-        if (tc_trtri)
-            REALQ_TRY(tc_trans_planes(rs, kb, n - k0, U + k0 * n + k0, n, UTh + k0 * n + k0, UTl + k0 * n + k0, n));
-    }
-    if (aux) {
-        REALQ_CUDA_TRY(cudaEventRecord(aux->ev[1], rs));
-        REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->ev[1], 0));
-        // join the wide stream only if it forked from s (under stream capture
-        // a wait on an event recorded outside the capture is an error)
-        if (wide_used) {
-            REALQ_CUDA_TRY(cudaEventRecord(aux->ev[2], aux->wide));
-            REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->ev[2], 0));
-        }
-    }
+    if (n <= PB)
+        REALQ_TRY(chol_inv_block(s, n, U, n, 0, status));
+    else if (ws_bytes >= prepare_ws_bytes(n))
+        REALQ_TRY(prepare_blocked(s, n, U, status, status_tc, static_cast<unsigned char *>(ws) + prepare_bytes(n),
+                                  overlap));
+    else
+        REALQ_TRY(prepare_steps(s, n, U, Vd, panel, status));
     if (!sync) return REALQ_OK;  // the failing column stays in the workspace's first word
     int host_status[2] = {-1, 0};
     REALQ_CUDA_TRY(cudaMemcpyAsync(host_status, status, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
