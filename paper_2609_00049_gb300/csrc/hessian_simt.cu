@@ -6,6 +6,7 @@
 // are reduced in a fixed order (bitwise repeatable).
 #include "kernels.cuh"
 
+#include <algorithm>
 #include <cmath>
 
 namespace realq {
@@ -179,8 +180,6 @@ realq_status_t hessian_reduce(cudaStream_t s, int64_t n, int splits, const float
 }
 
 int hessian_splits(int64_t n, int64_t T, int sms) {
-    // tiles of the tensor-core symmetric product: 128-channel row blocks by
-    // 256-channel column blocks reaching the diagonal
     const int nti = ceil_div(n, 128);
     int64_t tiles = 0;
     for (int r = 0; r < nti; ++r) tiles += r / 2 + 1;
@@ -211,8 +210,8 @@ int hessian_splits_tiles(int64_t tiles, int64_t T, int sms) {
 size_t hessian_ws_bytes(int64_t n, int64_t T, int has_xfp) {
     size_t b = align_up(sizeof(int));
     const int splits = hessian_splits(n, T, 152);
-    if (splits > 1) b += (size_t)splits * n * n * sizeof(float) * (has_xfp ? 2 : 1);
-    return b;
+    const size_t simt = splits > 1 ? (size_t)splits * n * n * sizeof(float) * (has_xfp ? 2 : 1) : 0;
+    return b + std::max(simt, hessian_tc_ws_bytes(n, T, has_xfp != 0, 152));
 }
 
 realq_status_t hessian_accumulate(cudaStream_t s, int64_t n, int64_t T, const void *X, const void *Xfp,
@@ -228,9 +227,10 @@ realq_status_t hessian_accumulate(cudaStream_t s, int64_t n, int64_t T, const vo
     }
     const bool tc_path = dt == REALQ_BF16 && hessian_tc_eligible(n, T, X);
     const bool tc_cross = tc_path && Xfp && hessian_tc_eligible(n, T, Xfp);
-    // tensor cores: H += X̂ᵀX̂ (and D += X̂ᵀX̂ from the same pass), D -= XᵀX̂
-    if (tc_path) REALQ_TRY(hessian_syrk_tc(s, n, T, X, H, err, pw, pbytes, num_sms(), tc_cross ? D : nullptr));
-    if (tc_cross) REALQ_TRY(hessian_cross_tc(s, n, T, Xfp, X, D, -1.f, err, pw, pbytes, num_sms()));
+    // tensor cores: H += X̂ᵀX̂ and D += X̂ᵀX̂ - XᵀX̂
+    if (tc_path)
+        REALQ_TRY(hessian_syrk_tc(s, n, T, X, tc_cross ? Xfp : nullptr, H, tc_cross ? D : nullptr, err, pw, pbytes,
+                                  num_sms()));
     float *Hs = tc_path ? nullptr : H;
     if (tc_cross) {
         Xfp = nullptr;

@@ -1,87 +1,96 @@
 // Step a2 (Sec. 3.2) on the 5th-generation tensor cores: H_sum += X̂^T X̂ for
 // bf16 calibration activations.
 //
-// One CTA owns one 128 x 256 tile (128 channels i by 256 channels j, on or
-// below the diagonal at 128-channel granularity) of H and a contiguous range
-// of tokens.  X̂ is token-major (T x n), so both MMA operands are read
-// MN-major straight from the activation rows: a TMA box of 64 tokens x 64
-// channels (128-byte rows, 128-byte swizzle) is one canonical MN-major atom
-// stack; two boxes make the 128-channel A operand and four the 256-channel B
-// operand (LBO = 8 KB between boxes, SBO = 1 KB between 8-token groups), and
-// one tcgen05.mma of M = 128, N = 256, K = 16 covers a 16-token step.  The
-// wide tile halves the A traffic per flop and lets a 4-stage, 192 KB ring
-// cover twice the MMA time of a 128 x 128 tile's.
+// A pair of CTAs (a cluster of two, cta_group::2) owns one 256 x 256 tile (256
+// channels i by 256 channels j, on or below the diagonal) of H and a contiguous
+// range of tokens; each CTA loads its 128 channels of A and its 128 channels of
+// B, the leader issues tcgen05.mma of M = 256, N = 256, K = 16 for both, and each
+// CTA's TMEM takes its own 128 rows.  X̂ is token-major (T x n), so both MMA
+// operands are read MN-major straight from the activation rows: a TMA box of 64
+// tokens x 64 channels (128-byte rows, 128-byte swizzle) is one canonical
+// MN-major atom stack; two boxes make a CTA's 128 channels of an operand (LBO =
+// 8 KB between boxes, SBO = 1 KB between 8-token groups).
+//
+// What bounds it: a 128 x 256 tile per CTA reads 12 KB of shared memory per MMA
+// of 128 cycles and is written 48 KB per four of them, 192 bytes per cycle
+// against the 128 that an SM serves, so it topped out at two thirds of the
+// tensor pipe.  The pair halves B's share: 64 + 64 bytes per cycle.
 //
 // Precision: the tensor core's fp32 accumulation loses about one unit in the
 // last place per accumulated MMA, in one direction, so a TMEM accumulator that
 // takes all 2^18 tokens of a calibration set (2^14 MMAs) drifts by ~1e-3 of
 // the entry.  The accumulation is therefore promoted: TMEM holds two 128 x 256
-// accumulators, the MMA issuer switches between them every 1024 tokens, and
+// accumulators (per CTA), the MMA issuer switches between them every 1024 tokens (512 halve the error but cost 6 %), and
 // the eight drain warps add each finished chunk into fp32 registers (IEEE
 // adds) while the other accumulator fills.
 //
-// Roles (320 threads): warp 8 lane 0 issues TMA into a STAGES-deep ring,
-// warp 9 lane 0 issues the MMAs and frees stages with tcgen05.commit; warps
-// 0-7 drain the accumulators (warp w owns TMEM lanes 32 (w % 4).. and columns
-// 128 (w / 4)..) and finally add their piece to H (mirrored below the
-// diagonal block), or store it as a partial sum when tokens are split.
-// The cross mode computes the full (non-symmetric) product X_Aᵀ X_B of two
-// token-major inputs over all tiles, scaled by a sign and added to the output
-// without mirroring: the cross moment of the perturbed-input surrogate is
-// D = X̂ᵀX̂ - XᵀX̂, the symmetric pass (also added into D) minus this one.
+// Roles (320 threads per CTA): warp 8 lane 0 issues the CTA's TMA loads into a
+// STAGES-deep ring (counted on the leader's barriers), warp 9 lane 0 of the
+// leader issues the MMAs and frees the stages of both CTAs with
+// tcgen05.commit; warps 0-7 drain the CTA's accumulators (warp w owns TMEM
+// lanes 32 (w % 4).. and columns 128 (w / 4)..) and finally add their piece to H
+// (mirrored below the diagonal block), or store it as a partial sum when tokens
+// are split; either way through a shared-memory block, so that a row's accesses
+// coalesce (one row per thread cost 40 us at n = 1024).
+//
+// A width that is no multiple of 256 leaves a last block of n % 256 channels.
+// Its tiles take it as the columns (the MMA's N, down to 32), also where it
+// belongs on the rows: such a tile is computed transposed ("swap") and stored
+// so.  At n = 2056 the last block's tiles are 26 of 126 and cost 0.3 of a full
+// one each.
+//
+// The cross tiles compute the full (non-symmetric) product X_Cᵀ X_B: the cross
+// moment of the perturbed-input surrogate is D = X̂ᵀX̂ - XᵀX̂.  With token splits
+// both products run in one launch over the same splits and the reduction
+// subtracts their sums (kept in two floats each) before it adds to D, so that
+// little of D is lost to the size of its two parts; without splits the
+// symmetric pass also adds into D and a second launch subtracts.
 // Every wait is bounded; on a timeout the tile is written as NaN (so the
 // factorisation of H reports a non-finite pivot), the workspace status word
 // gets ST_TIMEOUT, and the kernel still frees TMEM and returns.
 #include "kernels.cuh"
 #include "tc.cuh"
 
+#include <algorithm>
+#include <cmath>
 #include <mutex>
+#include <type_traits>
 
 namespace realq {
 namespace {
 
-constexpr int TM = 128;                          // tile rows (channels i)
-constexpr int TN = 256;                          // tile columns (channels j)
+constexpr int TM = 128;                          // tile rows of one CTA (channels i)
+constexpr int TN = 256;                          // tile rows of the pair, and tile columns (channels j)
 constexpr int KSTAGE = 64;                       // tokens per pipeline stage
-constexpr int STAGES = 4;
+constexpr int STAGES = 6;
 constexpr int CHUNK_STAGES = 16;                 // default: 1024 tokens per TMEM accumulator pass
 constexpr int DRAIN_WARPS = 8;                   // two per TMEM lane quarter, 128 columns each
 constexpr int THREADS = (DRAIN_WARPS + 2) * 32;  // + the TMA warp and the MMA warp
 constexpr int BOX_BYTES = 64 * KSTAGE * 2;       // one TMA box (64 channels x 64 tokens)
 constexpr int A_BYTES = TM * KSTAGE * 2;         // 2 boxes
-constexpr int B_BYTES = TN * KSTAGE * 2;         // 4 boxes
+constexpr int B_BYTES = TM * KSTAGE * 2;         // 2 boxes: this CTA's half of the columns
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
-constexpr uint32_t IDESC = tc::idesc_bf16_f32(TM, TN, 1, 1);
 constexpr unsigned FULL = 0xFFFFFFFFu;
 
-// Tiles of the symmetric product: row block ti (128 channels) with every
-// 256-wide column block tj that reaches the diagonal (256 tj <= 128 ti).
-__host__ __device__ inline int64_t lower_tiles(int nti) {
-    int64_t c = 0;
-    for (int r = 0; r < nti; ++r) c += r / 2 + 1;
-    return c;
-}
-
-// The lower tiles in groups of 8 row blocks: a group's tiles column by
-// column (within a column, its rows that reach it), so that the CTAs resident
-// at one time cover a compact block of the product and share their channel
-// blocks through L2.  A bijection onto {(ti, tj): tj <= ti / 2, ti < nti}.
-__device__ __forceinline__ void lower_tile(int64_t idx, int nti, int &ti, int &tj) {
-    constexpr int G = 8;
+// The lower tiles (ti >= tj of nt x nt) in groups of 4 tile rows: a group's tiles
+// column by column (within a column, its rows that reach it), so that the CTAs
+// resident at one time cover a compact block of the product and share their
+// channel blocks through L2.  A bijection onto {(ti, tj): tj <= ti < nt}.
+__device__ __forceinline__ void lower_tile(int64_t idx, int nt, int &ti, int &tj) {
+    constexpr int G = 4;
     int r0 = 0;
     for (;; r0 += G) {
-        const int r1 = min(r0 + G, nti);
-        int64_t c = 0;
-        for (int r = r0; r < r1; ++r) c += r / 2 + 1;
-        if (idx < c || r1 >= nti) break;
+        const int r1 = min(r0 + G, nt);
+        const int64_t c = (int64_t)r1 * (r1 + 1) / 2 - (int64_t)r0 * (r0 + 1) / 2;
+        if (idx < c || r1 >= nt) break;
         idx -= c;
     }
-    const int r1 = min(r0 + G, nti);
+    const int r1 = min(r0 + G, nt);
     for (int j = 0;; ++j) {
-        const int lo = max(r0, 2 * j);
+        const int lo = max(r0, j);
         const int cnt = r1 > lo ? r1 - lo : 0;
-        if (cnt == 0) {   // (not reached for idx < lower_tiles(nti))
+        if (cnt == 0) {   // (not reached for idx < nt (nt + 1) / 2)
             ti = r1 - 1;
             tj = 0;
             return;
@@ -95,29 +104,81 @@ __device__ __forceinline__ void lower_tile(int64_t idx, int nti, int &ti, int &t
     }
 }
 
+// A tile of the launch: A's 256-channel block ti, B's block tj with ncol (32 ..
+// 256) columns; cross or symmetric; swap: stored transposed.
+struct HessTile {
+    int ti, tj, ncol;
+    bool cross, swap;
+};
+struct HessGrid {
+    int64_t n;
+    int nf, rem;           // full 256-channel blocks, channels of the last one
+    int64_t nsym, ncross;  // tiles
+};
+inline HessGrid hess_grid(int64_t n, bool sym, bool cross) {
+    HessGrid g{n, (int)(n / TN), (int)(n % TN), 0, 0};
+    const int64_t r = g.rem ? 1 : 0, nf = g.nf;
+    if (sym) g.nsym = nf * (nf + 1) / 2 + r * (nf + 1);
+    if (cross) g.ncross = nf * nf + r * (2 * nf + 1);
+    return g;
+}
+__device__ __forceinline__ HessTile hess_tile(const HessGrid &g, int64_t idx) {
+    HessTile t{0, 0, TN, false, false};
+    const int nlast = (g.rem + 31) / 32 * 32;
+    if (idx < g.nsym) {
+        const int64_t full = (int64_t)g.nf * (g.nf + 1) / 2;
+        if (idx < full) {
+            lower_tile(idx, g.nf, t.ti, t.tj);
+        } else {
+            t.ti = (int)(idx - full);
+            t.tj = g.nf;
+            t.ncol = nlast;
+            t.swap = t.ti < g.nf;
+        }
+        return t;
+    }
+    idx -= g.nsym;
+    t.cross = true;
+    const int64_t full = (int64_t)g.nf * g.nf;
+    if (idx < full) {
+        // groups of 4 tile rows, column by column
+        constexpr int G = 4;
+        const int64_t per = (int64_t)G * g.nf;
+        const int r0 = (int)(idx / per) * G, gm = min(G, g.nf - r0);
+        t.ti = r0 + (int)(idx % per) % gm;
+        t.tj = (int)((idx % per) / gm);
+        return t;
+    }
+    idx -= full;
+    t.tj = g.nf;
+    t.ncol = nlast;
+    t.swap = idx > g.nf;                                     // (the last row block's other tiles)
+    t.ti = (int)(t.swap ? idx - g.nf - 1 : idx);
+    return t;
+}
+
 __global__ void __launch_bounds__(THREADS, 1)
-    hess_tc_kernel(const __grid_constant__ CUtensorMap tmap, const __grid_constant__ CUtensorMap tmapB, int64_t n,
-                   int64_t T, int64_t tper, float *H, float *H2, float *part, int direct, int cross, int two_maps,
-                   float sign, int chunk_stages, int *err) {
+    hess_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                   const __grid_constant__ CUtensorMap mapC, const HessGrid grid, int64_t T, int64_t tper, float *H,
+                   float *H2, float *part, float *partC, float sign, int chunk_stages, int *err) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + STAGES * STAGE_BYTES);
     uint64_t *empty = full + STAGES;
     uint64_t *accf = empty + STAGES;             // [2] accumulator b holds a finished chunk
     uint64_t *acce = accf + 2;                   // [2] accumulator b has been drained
-    uint32_t *tslot = reinterpret_cast<uint32_t *>(acce + 2);
+    uint64_t *drain = acce + 2;                  // the MMA thread's last commit
+    uint32_t *tslot = reinterpret_cast<uint32_t *>(drain + 1);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tslot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nti = (int)((n + TM - 1) / TM), ntj = (int)((n + TN - 1) / TN);
-    int ti, tj;
-    if (cross) {
-        ti = (int)(blockIdx.x / ntj);
-        tj = (int)(blockIdx.x % ntj);
-    } else {
-        lower_tile(blockIdx.x, nti, ti, tj);
-    }
-    const int i0 = ti * TM, j0 = tj * TN;
+    const int64_t n = grid.n;
+    const uint32_t rank = tc::cluster_rank();
+    const bool leader = rank == 0;
+    const HessTile tl = hess_tile(grid, blockIdx.x / 2);
+    // this CTA's 128 rows of the tile, and its half of the columns as an operand
+    const int i0 = tl.ti * TN + (int)rank * TM, jl = tl.tj * TN + (int)rank * (tl.ncol / 2);
+    const int bboxes = (tl.ncol / 2 + 63) / 64;
     const int64_t t_begin = (int64_t)blockIdx.y * tper;
     const int64_t t_end = min(T, t_begin + tper);
     const int nk = t_end > t_begin ? (int)((t_end - t_begin + KSTAGE - 1) / KSTAGE) : 0;
@@ -130,16 +191,19 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         for (int b = 0; b < 2; ++b) {
             tc::mbar_init(tc::smem_u32(&accf[b]), 1);
-            tc::mbar_init(tc::smem_u32(&acce[b]), DRAIN_WARPS);
+            tc::mbar_init(tc::smem_u32(&acce[b]), 2 * DRAIN_WARPS);   // both CTAs' (the leader's is waited on)
         }
+        tc::mbar_init(tc::smem_u32(drain), 1);
         *abort_flag = 0;
         tc::fence_barrier_init();
-        tc::prefetch_tmap(&tmap);
-        if (two_maps) tc::prefetch_tmap(&tmapB);
+        tc::prefetch_tmap(&mapA);
+        tc::prefetch_tmap(&mapB);
+        tc::prefetch_tmap(&mapC);
     }
-    if (warp == 0) tc::tmem_alloc(tc::smem_u32(tslot), 2 * TN);
+    if (warp == 0) tc::tmem_alloc_pair(tc::smem_u32(tslot), 2 * TN);
     tc::fence_before_sync();
     __syncthreads();
+    tc::cluster_sync();   // the peer's barriers are initialized
     tc::fence_after_sync();
     const uint32_t tmem = *tslot;
 
@@ -151,7 +215,10 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (warp == DRAIN_WARPS) {
         if (lane == 0) {
             // ---------------- TMA producer ----------------
-            const CUtensorMap *mb = two_maps ? &tmapB : &tmap;
+            // symmetric: A from mapA, B from mapB; cross: A from mapC, B from
+            // mapB, the other way round when the tile is stored transposed
+            const CUtensorMap *ma = !tl.cross ? &mapA : (tl.swap ? &mapB : &mapC);
+            const CUtensorMap *mb = tl.cross && tl.swap ? &mapC : &mapB;
             int it = 0;
             for (; it < nk; ++it) {
                 const int s = it % STAGES;
@@ -160,17 +227,18 @@ __global__ void __launch_bounds__(THREADS, 1)
                     *abort_flag = 1;
                     break;
                 }
-                const uint32_t fb = tc::smem_u32(&full[s]);
-                tc::mbar_arrive_expect_tx(fb, STAGE_BYTES);
+                // (both CTAs' bytes are counted on the leader's barrier)
+                const uint32_t fb = tc::mapa(tc::smem_u32(&full[s]), 0);
+                if (leader) tc::mbar_arrive_expect_tx(tc::smem_u32(&full[s]), 2 * (A_BYTES + bboxes * BOX_BYTES));
                 const int y = (int)(t_begin + (int64_t)it * KSTAGE);
                 const uint32_t a = tc::smem_u32(smem + s * STAGE_BYTES);
-                tc::tma_load_2d(a, &tmap, fb, i0, y);
-                tc::tma_load_2d(a + BOX_BYTES, &tmap, fb, i0 + 64, y);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) tc::tma_load_2d(a + A_BYTES + q * BOX_BYTES, mb, fb, j0 + 64 * q, y);
+                tc::tma_load_2d_pair(a, ma, fb, i0, y);
+                tc::tma_load_2d_pair(a + BOX_BYTES, ma, fb, i0 + 64, y);
+                for (int q = 0; q < bboxes; ++q) tc::tma_load_2d_pair(a + A_BYTES + q * BOX_BYTES, mb, fb, jl + 64 * q, y);
             }
-            // on abort, let the copies already issued land before the CTA exits
-            if (*abort_flag) {
+            // on abort, let the copies already issued land before the CTAs
+            // exit (the leader waits for both, before the cluster barrier)
+            if (*abort_flag && leader) {
                 int never = 0;
                 for (int k = (it > STAGES ? it - STAGES : 0); k < it; ++k)
                     tc::mbar_wait(tc::smem_u32(&full[k % STAGES]), (uint32_t)(k / STAGES) & 1u, &never,
@@ -178,8 +246,9 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
         }
     } else if (warp == DRAIN_WARPS + 1) {
-        if (lane == 0) {
+        if (lane == 0 && leader) {
             // ---------------- MMA issuer ----------------
+            const uint32_t idesc = tc::idesc_bf16_f32(2 * TM, (uint32_t)tl.ncol, 1, 1);
             for (int c = 0; c < nch && !*abort_flag; ++c) {
                 const int b = c & 1;
                 if (c >= 2 && !tc::mbar_wait(tc::smem_u32(&acce[b]), (uint32_t)((c >> 1) - 1) & 1u, abort_flag)) {
@@ -204,17 +273,21 @@ __global__ void __launch_bounds__(THREADS, 1)
                     for (int k = 0; k < KSTAGE / 16; ++k) {
                         const uint64_t da = tc::smem_desc(a + k * 2048, BOX_BYTES, 1024, tc::SW_128B);
                         const uint64_t db = tc::smem_desc(bop + k * 2048, BOX_BYTES, 1024, tc::SW_128B);
-                        tc::mma_bf16_ss(d, da, db, IDESC, (first && k == 0) ? 0u : 1u);
+                        tc::mma_f16_pair(d, da, db, idesc, (first && k == 0) ? 0u : 1u);
                     }
-                    tc::mma_commit(tc::smem_u32(&empty[s]));
+                    tc::mma_commit_pair(tc::smem_u32(&empty[s]));
                 }
-                tc::mma_commit(tc::smem_u32(&accf[b]));
+                tc::mma_commit_pair(tc::smem_u32(&accf[b]));
             }
+            // every MMA issued has retired before TMEM is freed
+            tc::mma_commit_pair(tc::smem_u32(drain));
+            int never = 0;
+            tc::mbar_wait(tc::smem_u32(drain), 0u, &never, 100000000ull);
         }
     } else {
         // ------- drain warps: TMEM chunk -> fp32 registers (lane quarter, column half) -------
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t col_base = (uint32_t)((warp >> 2) * 128);
+        const int col_base = (warp >> 2) * 128;
         for (int c = 0; c < nch; ++c) {
             const int b = c & 1;
             const bool ok = tc::mbar_wait(tc::smem_u32(&accf[b]), (uint32_t)(c >> 1) & 1u, abort_flag);
@@ -224,64 +297,78 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
             tc::fence_after_sync();
 #pragma unroll
-            for (int c0 = 0; c0 < 128; c0 += 32) {
-                uint32_t v[32];
-                tc::tmem_ld_32x32b_x32(tmem + lane_base + (uint32_t)(b * TN) + col_base + (uint32_t)c0, v);
+            for (int c0 = 0; c0 < 128; c0 += 16) {
+                if (col_base + c0 < tl.ncol) {
+                    uint32_t v[16];
+                    tc::tmem_ld_32x32b_x16(tmem + lane_base + (uint32_t)(b * TN + col_base + c0), v);
 #pragma unroll
-                for (int q = 0; q < 32; ++q) acc[c0 + q] += __uint_as_float(v[q]);
+                    for (int q = 0; q < 16; ++q) acc[c0 + q] += __uint_as_float(v[q]);
+                }
             }
             tc::fence_before_sync();
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive(tc::smem_u32(&acce[b]));
+            if (lane == 0) tc::mbar_arrive_cluster(tc::mapa(tc::smem_u32(&acce[b]), 0));
         }
     }
     __syncwarp();
     const bool all_good = __syncthreads_and(good && !*abort_flag) != 0;
 
-    // ---------------- epilogue: registers -> global (drain warps) ----------------
-    // Each drain warp owns a 32-row x 128-column piece, in 128-column block
-    // jb of the matrix.  Symmetric product: jb < ti is added and mirrored,
-    // jb == ti (the diagonal block) is added in full, jb > ti lies above the
-    // diagonal and is left to the tile that holds its mirror image.
-    if (warp < DRAIN_WARPS) {
-        const int jb = 2 * tj + (warp >> 2);
-        const bool write = cross || jb <= ti;
-        const bool mirror = !cross && jb < ti;
-        const int64_t gi = i0 + (warp & 3) * 32 + lane;
-        const int64_t gj0 = (int64_t)jb * 128;
-        if (write && gi < n) {
-            if (!all_good) {
-                // poison: the factorisation of H then reports a non-finite pivot
-                for (int q = 0; q < 128 && gj0 + q < n; ++q) {
-                    const int64_t gj = gj0 + q;
-                    if (direct) {
-                        H[gi * n + gj] = __int_as_float(0x7fc00000);
-                        if (mirror) H[gj * n + gi] = __int_as_float(0x7fc00000);
-                        if (H2) {
-                            H2[gi * n + gj] = __int_as_float(0x7fc00000);
-                            if (mirror) H2[gj * n + gi] = __int_as_float(0x7fc00000);
-                        }
-                    } else {
-                        part[(int64_t)blockIdx.y * n * n + gi * n + gj] = __int_as_float(0x7fc00000);
+    // ---------------- epilogue (drain warps) ----------------
+    // Each drain warp owns a 32-row x 128-column piece, in 128-row block ib and
+    // 128-column block jb of the matrix.  Symmetric product: jb < ib is added
+    // and mirrored, jb == ib (the diagonal block) is added in full, jb > ib lies
+    // above the diagonal and is left to the CTA that holds its mirror image (a
+    // swapped tile lies above it as a whole and is added mirrored).
+    if (warp < DRAIN_WARPS && (nk > 0 || !all_good)) {
+        const bool direct = part == nullptr;
+        const int ib = 2 * tl.ti + (int)rank, jb = 2 * tl.tj + (warp >> 2);
+        const bool plain = tl.cross ? !tl.swap : (tl.swap ? direct : jb <= ib);              // at [i][j]
+        const bool turned = tl.cross ? tl.swap : (tl.swap || (direct && jb < ib));           // at [j][i]
+        const float mul = tl.cross ? sign : 1.f;
+        float *o1 = direct ? H : (tl.cross ? partC : part) + (int64_t)blockIdx.y * n * n;
+        float *o2 = direct && !tl.cross ? H2 : nullptr;
+        float *st = reinterpret_cast<float *>(smem) + warp * 32 * 33;
+        const int64_t gi0 = i0 + (warp & 3) * 32, gi = gi0 + lane;
+#pragma unroll
+        for (int c0 = 0; c0 < 128; c0 += 32) {
+            const int64_t gj0 = (int64_t)tl.tj * TN + (warp >> 2) * 128 + c0;
+            if (gj0 >= n || gi0 >= n) continue;
+            float v[32];
+#pragma unroll
+            for (int q = 0; q < 32; ++q) v[q] = all_good ? mul * acc[c0 + q] : __int_as_float(0x7fc00000);
+#pragma unroll 1
+            for (int w = 0; w < 2; ++w) {
+                float *o = w ? o2 : o1;
+                if (!o) break;
+                if (turned && gi < n) {
+                    float *d = o + gj0 * n + gi;
+#pragma unroll
+                    for (int h = 0; h < 32; h += 16) {
+                        float old[16];
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) old[q] = direct && gj0 + h + q < n ? d[(h + q) * n] : 0.f;
+#pragma unroll
+                        for (int q = 0; q < 16; ++q)
+                            if (gj0 + h + q < n) d[(h + q) * n] = old[q] + v[h + q];
                     }
                 }
-            } else if (nk > 0) {
+                if (plain) {
 #pragma unroll
-                for (int q = 0; q < 128; ++q) {
-                    const int64_t gj = gj0 + q;
-                    if (gj < n) {
-                        const float v = sign * acc[q];
-                        if (direct) {
-                            H[gi * n + gj] += v;
-                            if (mirror) H[gj * n + gi] += v;
-                            if (H2) {
-                                H2[gi * n + gj] += v;
-                                if (mirror) H2[gj * n + gi] += v;
-                            }
-                        } else {
-                            part[(int64_t)blockIdx.y * n * n + gi * n + gj] = v;
+                    for (int q = 0; q < 32; ++q) st[lane * 33 + q] = v[q];
+                    __syncwarp();
+                    if (gj0 + lane < n) {
+                        float *d = o + gi0 * n + gj0 + lane;
+#pragma unroll 1
+                        for (int h = 0; h < 32; h += 16) {
+                            float old[16];
+#pragma unroll
+                            for (int q = 0; q < 16; ++q) old[q] = direct && gi0 + h + q < n ? d[(h + q) * n] : 0.f;
+#pragma unroll
+                            for (int q = 0; q < 16; ++q)
+                                if (gi0 + h + q < n) d[(h + q) * n] = old[q] + st[(h + q) * 33 + lane];
                         }
                     }
+                    __syncwarp();
                 }
             }
         }
@@ -289,7 +376,93 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (!all_good && threadIdx.x == 0 && err) atomicOr(err, ST_TIMEOUT);
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tmem, 2 * TN);
+    tc::cluster_sync();   // neither CTA leaves while the other may signal its barriers
+    if (warp == 0) tc::tmem_dealloc_pair(tmem, 2 * TN);
+}
+
+// s += a with the rounding error kept in e
+__device__ __forceinline__ void two_sum(float &s, float &e, float a) {
+    const float t = s + a, z = t - s;
+    e += (s - (t - z)) + (a - z);
+    s = t;
+}
+
+// H += the symmetric partial sums over the splits, mirrored, and with D also
+// D += symmetric - cross partial sums.  One CTA per TILE x TILE tile (bi >= bj)
+// of the lower triangle, four columns per thread with all splits' loads in
+// flight; the mirror image goes through shared memory, so that every access is
+// part of a row of float4 (n a multiple of 8).  Sums carry their rounding
+// error: D is the small difference of two large sums.  MS bounds the splits (4,
+// 8 or 16), so that few splits take few registers.
+constexpr int MAX_SPLITS = 16;
+template <bool CROSS, int MS, int TILE>
+__global__ void __launch_bounds__(256) hess_tc_reduce_kernel(int64_t n, int splits, const float *part,
+                                                             const float *partC, float *H, float *D) {
+    constexpr int TPR = TILE / 4, ROWS = 256 / TPR, PER = TILE / ROWS;   // threads per row, rows per pass, passes
+    __shared__ float th[TILE][TILE + 1], tl[TILE][TILE + 1];
+    int bi = (int)((sqrt(8.0 * (double)blockIdx.x + 1.0) - 1.0) * 0.5);
+    while ((int64_t)(bi + 1) * (bi + 2) / 2 <= blockIdx.x) ++bi;
+    while ((int64_t)bi * (bi + 1) / 2 > blockIdx.x) --bi;
+    const int bj = (int)(blockIdx.x - (int64_t)bi * (bi + 1) / 2);
+    const int r0 = threadIdx.x / TPR, c = (threadIdx.x % TPR) * 4;
+    const int64_t nn = n * n;
+    auto sum = [&](const float *p, float (&s)[4], float (&e)[4]) {
+        float4 v[MS];
+#pragma unroll
+        for (int k = 0; k < MS; ++k)
+            if (k < splits) v[k] = *reinterpret_cast<const float4 *>(p + k * nn);
+#pragma unroll
+        for (int k = 0; k < MS; ++k)
+            if (k < splits) {
+                two_sum(s[0], e[0], v[k].x); two_sum(s[1], e[1], v[k].y);
+                two_sum(s[2], e[2], v[k].z); two_sum(s[3], e[3], v[k].w);
+            }
+    };
+    auto add = [&](int64_t at, const float (&s)[4], const float (&e)[4]) {
+        if (CROSS) {
+            float x[4] = {}, xe[4] = {};
+            sum(partC + at, x, xe);
+            float4 d = *reinterpret_cast<const float4 *>(D + at);
+            d.x += (s[0] - x[0]) + (e[0] - xe[0]);
+            d.y += (s[1] - x[1]) + (e[1] - xe[1]);
+            d.z += (s[2] - x[2]) + (e[2] - xe[2]);
+            d.w += (s[3] - x[3]) + (e[3] - xe[3]);
+            *reinterpret_cast<float4 *>(D + at) = d;
+        }
+        float4 h = *reinterpret_cast<const float4 *>(H + at);
+        h.x += s[0] + e[0]; h.y += s[1] + e[1]; h.z += s[2] + e[2]; h.w += s[3] + e[3];
+        *reinterpret_cast<float4 *>(H + at) = h;
+    };
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int r = r0 + u * ROWS;
+        const int64_t i = (int64_t)bi * TILE + r, j = (int64_t)bj * TILE + c;
+        float s[4] = {}, e[4] = {};
+        if (i < n && j < n) {
+            sum(part + i * n + j, s, e);
+            add(i * n + j, s, e);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            th[r][c + q] = s[q];
+            tl[r][c + q] = e[q];
+        }
+    }
+    if (bi == bj) return;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int r = r0 + u * ROWS;
+        const int64_t i = (int64_t)bj * TILE + r, j = (int64_t)bi * TILE + c;
+        if (i >= n || j >= n) continue;
+        float s[4], e[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            s[q] = th[c + q][r];
+            e[q] = tl[c + q][r];
+        }
+        add(i * n + j, s, e);
+    }
 }
 
 using EncodeFn = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -367,55 +540,123 @@ bool hessian_tc_eligible(int64_t n, int64_t T, const void *X) {
            n < (1ll << 31);
 }
 
-// out (+= sign X_Aᵀ X_B); symmetric (X_B null): lower tiles mirrored, and
-// out2 (if given) receives the same sum.  Token splits go through the
-// workspace partials and a fixed-order reduction.
-static realq_status_t hess_tc_launch(cudaStream_t s, int64_t n, int64_t T, const void *XA, const void *XB, float *out,
-                                     float *out2, float sign, int *err, void *ws, size_t ws_bytes, int sms,
-                                     const char *name, int chunk_stages = CHUNK_STAGES, bool sym_pair = false) {
-    CUtensorMap mapA, mapB;
-    CUresult cr = encode_tmap_2d_bf16(&mapA, XA, (uint64_t)n, (uint64_t)T, (uint64_t)n * 2, 64, KSTAGE, 1);
-    if (cr == CUDA_SUCCESS && XB)
-        cr = encode_tmap_2d_bf16(&mapB, XB, (uint64_t)n, (uint64_t)T, (uint64_t)n * 2, 64, KSTAGE, 1);
+// Token splits of a launch of full (and 0.35 of a full one's time: last-block)
+// tiles over the pairs of SMs: the count that minimises rounds x (a split's
+// share of a tile's time + a CTA's fixed cost) + the partial sums' traffic,
+// in microseconds (a 64-token stage of a pair is 0.29 us at 1.75 GHz; a CTA's
+// start, fill and epilogue about 8 us; a partial 256 x 256 tile written and
+// read at 5 TB/s).  At least 1024 tokens per split (one promoted chunk) and at
+// most 16 splits.
+static int tc_splits(const HessGrid &g, int64_t T, int sms) {
+    const int64_t full = (g.nsym ? (int64_t)g.nf * (g.nf + 1) / 2 : 0) + (g.ncross ? (int64_t)g.nf * g.nf : 0);
+    const double tiles = (double)full + 0.35 * (double)(g.nsym + g.ncross - full);
+    const int pairs = sms / 2 > 0 ? sms / 2 : 1;
+    const int64_t most = std::min<int64_t>(MAX_SPLITS, std::max<int64_t>(1, T / 1024));
+    double best = 1e300;
+    int bs = 1;
+    for (int k = 1; k <= most; ++k) {
+        const double rounds = std::ceil(tiles * k / pairs - 1e-9);
+        const double us = rounds * ((double)T / 64.0 * 0.29 / k + 8.0) + (k > 1 ? k * tiles * 0.105 : 0.0);
+        if (us < best * (1.0 - 1e-9)) {
+            best = us;
+            bs = k;
+        }
+    }
+    return bs;
+}
+
+size_t hessian_tc_ws_bytes(int64_t n, int64_t T, bool cross, int sms) {
+    const int k = tc_splits(hess_grid(n, true, false), T, sms);
+    return k > 1 ? (size_t)k * n * n * sizeof(float) * (cross ? 2 : 1) : 0;
+}
+
+// H += X_Aᵀ X_B (symmetric; X_B null: X_A) when H is given, and D += sign (...):
+// with X_C, cross tiles X_Cᵀ X_B.  H and D with X_C: H += X_Aᵀ X_A, D += that
+// - X_Cᵀ X_A.
+static realq_status_t hess_tc_launch(cudaStream_t s, int64_t n, int64_t T, const void *XA, const void *XB,
+                                     const void *XC, float *H, float *D, int *err, void *ws, size_t ws_bytes, int sms,
+                                     const char *name, int chunk_stages) {
+    CUtensorMap mapA, mapB, mapC;
+    CUresult cr = CUDA_SUCCESS;
+    auto map = [&](CUtensorMap *m, const void *X) {
+        if (cr == CUDA_SUCCESS)
+            cr = encode_tmap_2d_bf16(m, X, (uint64_t)n, (uint64_t)T, (uint64_t)n * 2, 64, KSTAGE, 1);
+    };
+    map(&mapA, XA);
+    map(&mapB, XB ? XB : XA);
+    map(&mapC, XC ? XC : XA);
     if (cr != CUDA_SUCCESS) return fail(REALQ_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)cr);
-    if (!XB) mapB = mapA;
-    const int two_maps = XB != nullptr;
-    const int cross = two_maps && !sym_pair;
-    const int nti = ceil_div(n, TM), ntj = ceil_div(n, TN);
-    const int64_t tiles = cross ? (int64_t)nti * ntj : lower_tiles(nti);
-    int splits = hessian_splits_tiles(tiles, T, sms);
-    const size_t per = (size_t)n * n * sizeof(float);
+    const size_t per = (size_t)n * n * sizeof(float) * (XC ? 2 : 1);
+    // (the symmetric product's count also with cross tiles: H then has the same
+    // bits whether or not D is asked for)
+    int splits = tc_splits(hess_grid(n, true, false), T, sms);
     if (splits > 1 && (ws == nullptr || ws_bytes < 2 * per)) splits = 1;
-    if (splits > 1 && (size_t)splits * per > ws_bytes) splits = (int)(ws_bytes / per);
+    if (splits > 1 && (size_t)splits * per > ws_bytes) splits = (int)(ws_bytes / per);   // (at most the plan's)
     int64_t tper = (T + splits - 1) / splits;
     tper = (tper + KSTAGE - 1) / KSTAGE * KSTAGE;
     splits = (int)((T + tper - 1) / tper);
     REALQ_TRY(set_smem_limit(reinterpret_cast<const void *>(hess_tc_kernel), SMEM_BYTES));
-    float *part = static_cast<float *>(ws);
+    float *part = splits > 1 ? static_cast<float *>(ws) : nullptr;
+    float *partC = part ? part + (size_t)splits * n * n : nullptr;
+    auto launch = [&](const HessGrid &g, float *o, float *o2, float sign, const char *who) -> realq_status_t {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(2 * (g.nsym + g.ncross)), (unsigned)splits);
+        cfg.blockDim = dim3(THREADS);
+        cfg.dynamicSmemBytes = SMEM_BYTES;
+        cfg.stream = s;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 2;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        {
+            Launch L(who, s);
+            REALQ_CUDA_TRY(cudaLaunchKernelEx(&cfg, hess_tc_kernel, mapA, mapB, mapC, g, T, tper, o, o2, part, partC,
+                                              sign, chunk_stages, err));
+        }
+        return check_launch(who);
+    };
+    if (!part) {
+        // one split: straight into H and D
+        REALQ_TRY(launch(hess_grid(n, true, false), H, XC ? D : nullptr, 1.f, name));
+        if (XC) REALQ_TRY(launch(hess_grid(n, false, true), D, nullptr, -1.f, "hessian_cross_tc"));
+        return REALQ_OK;
+    }
+    REALQ_TRY(launch(hess_grid(n, true, XC != nullptr), nullptr, nullptr, 1.f, name));
+    // 64 x 64 tiles where they fill the SMs twice over, else 32 x 32 (n = 1024:
+    // 136 tiles took 24 us, 528 take 11)
+    const int tile = n >= 1536 ? 64 : 32;
+    const int64_t nb = ceil_div(n, tile);
+    const unsigned tiles = (unsigned)(nb * (nb + 1) / 2);
+    auto reduce = [&](auto cross, auto ms) {
+        constexpr bool CR = decltype(cross)::value;
+        constexpr int MS = decltype(ms)::value;
+        if (tile == 64) hess_tc_reduce_kernel<CR, MS, 64><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D);
+        else hess_tc_reduce_kernel<CR, MS, 32><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D);
+    };
+    auto by_splits = [&](auto cross) {
+        if (splits <= 4) reduce(cross, std::integral_constant<int, 4>());
+        else if (splits <= 8) reduce(cross, std::integral_constant<int, 8>());
+        else reduce(cross, std::integral_constant<int, MAX_SPLITS>());
+    };
     {
-        Launch L(name, s);
-        hess_tc_kernel<<<dim3((unsigned)tiles, (unsigned)splits), THREADS, SMEM_BYTES, s>>>(
-            mapA, mapB, n, T, tper, out, out2, part, splits == 1, cross, two_maps, sign, chunk_stages, err);
+        Launch L("hessian_reduce", s);
+        if (XC) by_splits(std::true_type());
+        else by_splits(std::false_type());
     }
-    REALQ_TRY(check_launch(name));
-    if (splits > 1) {
-        REALQ_TRY(hessian_reduce(s, n, splits, part, out, cross ? 1 : 0));
-        if (out2) REALQ_TRY(hessian_reduce(s, n, splits, part, out2, cross ? 1 : 0));
-    }
-    return REALQ_OK;
+    return check_launch("hessian_reduce");
 }
 
-realq_status_t hessian_syrk_tc(cudaStream_t s, int64_t n, int64_t T, const void *X, float *H, int *err, void *ws,
-                               size_t ws_bytes, int sms, float *H2) {
-    return hess_tc_launch(s, n, T, X, nullptr, H, H2, 1.f, err, ws, ws_bytes, sms, "hessian_syrk_tc");
+realq_status_t hessian_syrk_tc(cudaStream_t s, int64_t n, int64_t T, const void *X, const void *Xfp, float *H, float *D,
+                               int *err, void *ws, size_t ws_bytes, int sms) {
+    return hess_tc_launch(s, n, T, X, nullptr, Xfp, H, D, err, ws, ws_bytes, sms, "hessian_syrk_tc", CHUNK_STAGES);
 }
 
-realq_status_t hessian_cross_tc(cudaStream_t s, int64_t n, int64_t T, const void *XA, const void *XB, float *out,
-                                float sign, int *err, void *ws, size_t ws_bytes, int sms, int chunk_stages,
-                                bool symmetric) {
-    return hess_tc_launch(s, n, T, XA, XB, out, nullptr, sign, err, ws, ws_bytes, sms,
-                          symmetric ? "hessian_weighted_tc" : "hessian_cross_tc",
-                          chunk_stages > 0 ? chunk_stages : CHUNK_STAGES, symmetric);
+realq_status_t hessian_pair_tc(cudaStream_t s, int64_t n, int64_t T, const void *XA, const void *XB, float *H, int *err,
+                               void *ws, size_t ws_bytes, int sms, int chunk_stages) {
+    return hess_tc_launch(s, n, T, XA, XB, nullptr, H, nullptr, err, ws, ws_bytes, sms, "hessian_weighted_tc",
+                          chunk_stages);
 }
 
 }  // namespace realq

@@ -188,14 +188,15 @@ realq_status_t hessian_accumulate(cudaStream_t s, int64_t n, int64_t T, const vo
                                   realq_dtype_t dt, float *H, float *D, void *ws, size_t ws_bytes);
 realq_status_t hessian_reduce(cudaStream_t s, int64_t n, int splits, const float *part, float *out, int mode);
 bool hessian_tc_eligible(int64_t n, int64_t T, const void *X);
-realq_status_t hessian_syrk_tc(cudaStream_t s, int64_t n, int64_t T, const void *X, float *H, int *err, void *ws,
-                               size_t ws_bytes, int sms, float *H2 = nullptr);
-// out += sign X_Aᵀ X_B.  chunk_stages: 64-token stages per TMEM accumulator
-// pass before promotion (0: default).  symmetric: the product is known to be
-// symmetric (X_B = diag(s) X_A up to rounding): lower tiles only, mirrored.
-realq_status_t hessian_cross_tc(cudaStream_t s, int64_t n, int64_t T, const void *XA, const void *XB, float *out,
-                                float sign, int *err, void *ws, size_t ws_bytes, int sms, int chunk_stages = 0,
-                                bool symmetric = false);
+// H += X̂ᵀX̂, and with Xfp D += X̂ᵀX̂ - XfpᵀX̂
+realq_status_t hessian_syrk_tc(cudaStream_t s, int64_t n, int64_t T, const void *X, const void *Xfp, float *H, float *D,
+                               int *err, void *ws, size_t ws_bytes, int sms);
+// H += X_Aᵀ X_B where that is known to be symmetric (X_B = diag(s) X_A up to
+// rounding): lower tiles only, mirrored.  chunk_stages: 64-token stages per
+// TMEM accumulator pass before promotion.
+realq_status_t hessian_pair_tc(cudaStream_t s, int64_t n, int64_t T, const void *XA, const void *XB, float *H, int *err,
+                               void *ws, size_t ws_bytes, int sms, int chunk_stages);
+size_t hessian_tc_ws_bytes(int64_t n, int64_t T, bool cross, int sms);
 int hessian_splits_tiles(int64_t tiles, int64_t T, int sms);
 
 // --------------------------------------------------------------- prepare ---

@@ -159,8 +159,8 @@ realq_status_t hessian_weighted(cudaStream_t s, int64_t n, int64_t T, const void
         }
         REALQ_TRY(check_launch("saliency_scale"));
         float *Hout = Hg + (size_t)g * n * n;
-        REALQ_TRY(hessian_cross_tc(s, n, T, X, Yhi, Hout, 1.f, err, part, pbytes, num_sms(), kPromoteStages, true));
-        REALQ_TRY(hessian_cross_tc(s, n, T, X, Ylo, Hout, 1.f, err, part, pbytes, num_sms(), kPromoteStages, true));
+        REALQ_TRY(hessian_pair_tc(s, n, T, X, Yhi, Hout, err, part, pbytes, num_sms(), kPromoteStages));
+        REALQ_TRY(hessian_pair_tc(s, n, T, X, Ylo, Hout, err, part, pbytes, num_sms(), kPromoteStages));
     }
     {
         Launch L("saliency_wsum", s);

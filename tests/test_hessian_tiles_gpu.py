@@ -1,0 +1,32 @@
+"""The tensor-core Hessian and cross moment at the edges of their 256-channel
+tiles (a last block of 8 to 248 channels, computed as the columns of its tiles
+and stored transposed where it belongs on the rows), of the token stages and of
+the token splits, with and without room for the splits' partial sums.  Inputs
+are small integers, so that every sum is exact in fp32: equality."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2609_00049_gb300 as rq
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("splits", [True, False])
+@pytest.mark.parametrize("n,T", [(64, 1), (72, 100), (248, 1030), (256, 2049), (264, 5000), (384, 3000), (520, 9000),
+                                 (1000, 7777), (1288, 4096)])
+def test_exact_on_integers_at_tile_edges(n, T, splits):
+    g = torch.Generator().manual_seed(n + T)
+    Xh = torch.randint(-3, 4, (T, n), generator=g).to(torch.bfloat16).cuda()
+    Xf = torch.randint(-3, 4, (T, n), generator=g).to(torch.bfloat16).cuda()
+    ws = rq.workspace(rq.realq_hessian_workspace_size(n, T, rq.REALQ_BF16, True)) if splits else None
+    H0 = torch.randint(-5, 6, (n, n), generator=g).float().cuda()
+    H0 = H0 + H0.T
+    D0 = torch.randint(-5, 6, (n, n), generator=g).float().cuda()
+    H, D, P = H0.clone(), D0.clone(), H0.clone()
+    rq.realq_hessian_accumulate(Xh, H, D, Xf, ws=ws)
+    rq.realq_hessian_accumulate(Xh, P, ws=ws)
+    a, b = Xh.double().cpu(), Xf.double().cpu()
+    assert torch.equal(H.double().cpu(), H0.double().cpu() + a.T @ a)
+    assert torch.equal(D.double().cpu(), D0.double().cpu() + a.T @ a - b.T @ a)
+    assert torch.equal(P, H)
