@@ -8,6 +8,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 namespace realq {
 namespace {
@@ -106,6 +107,99 @@ __global__ void __launch_bounds__(THREADS) hess_kernel(int64_t n, int64_t T, con
     }
 }
 
+// The same product on 32 x 32 tiles, for inputs whose 128 x 128 tiles leave
+// most SMs idle (n = 512: 10 tiles took 382 us for 2048 tokens, 136 take 36).
+// Every element is the same sum over the tokens in order.  128 threads, four
+// rows by two columns each (bound by what shared memory delivers: 24 cycles per
+// token); 64 tokens are staged while the previous 64 are multiplied.
+constexpr int SB = 32, SK = 64, STHREADS = 128;
+__device__ __forceinline__ float4 ldx4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 ldx4(const __nv_bfloat16 *p) {
+    const uint2 u = *reinterpret_cast<const uint2 *>(p);
+    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xFFFF0000u), __uint_as_float(u.y << 16),
+                       __uint_as_float(u.y & 0xFFFF0000u));
+}
+
+template <typename TX, int MODE, bool VEC>
+__global__ void __launch_bounds__(STHREADS) hess_small_kernel(int64_t n, int64_t T, const TX *Xh, const TX *Xf,
+                                                              float *out, float *part, int64_t tper, int direct) {
+    __shared__ __align__(16) float As[2][SK][SB];
+    __shared__ __align__(16) float Bs[2][SK][SB];
+    const int nt = (int)((n + SB - 1) / SB);
+    int ti, tj;
+    tile_of(blockIdx.x, MODE == 0, nt, ti, tj);
+    const int64_t i0 = (int64_t)ti * SB, j0 = (int64_t)tj * SB;
+    const int64_t t_begin = (int64_t)blockIdx.y * tper;
+    const int64_t t_end = min(T, t_begin + tper);
+    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;      // columns 2 tx .., rows 4 ty ..
+    const int lr = tid >> 3, lc = (tid & 7) * 4;                     // staging: token row lr + 16 u, channels lc ..
+    float4 ra[SK / 16], rb[SK / 16];
+    auto at = [&](const TX *X, int64_t t, int64_t g0) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (t >= t_end) return v;
+        const TX *p = X + t * n + g0 + lc;
+        if (VEC && g0 + lc + 3 < n) return ldx4(p);
+        if (g0 + lc < n) v.x = ldx(p, 0);
+        if (g0 + lc + 1 < n) v.y = ldx(p, 1);
+        if (g0 + lc + 2 < n) v.z = ldx(p, 2);
+        if (g0 + lc + 3 < n) v.w = ldx(p, 3);
+        return v;
+    };
+    auto fetch = [&](int64_t t0) {
+#pragma unroll
+        for (int u = 0; u < SK / 16; ++u) {
+            const int64_t t = t0 + lr + 16 * u;
+            ra[u] = at(Xh, t, i0);
+            if (MODE == 1) {
+                const float4 f = at(Xf, t, i0);
+                ra[u].x -= f.x; ra[u].y -= f.y; ra[u].z -= f.z; ra[u].w -= f.w;
+            }
+            rb[u] = at(Xh, t, j0);
+        }
+    };
+    float acc[4][2] = {};
+    fetch(t_begin);
+    int b = 0;
+    for (int64_t t0 = t_begin; t0 < t_end; t0 += SK, b ^= 1) {
+#pragma unroll
+        for (int u = 0; u < SK / 16; ++u) {
+            *reinterpret_cast<float4 *>(&As[b][lr + 16 * u][lc]) = ra[u];
+            *reinterpret_cast<float4 *>(&Bs[b][lr + 16 * u][lc]) = rb[u];
+        }
+        __syncthreads();   // (the other buffer's readers passed this barrier a stage ago)
+        if (t0 + SK < t_end) fetch(t0 + SK);
+#pragma unroll 8
+        for (int k = 0; k < SK; ++k) {
+            const float4 a = *reinterpret_cast<const float4 *>(&As[b][k][ty * 4]);
+            const float2 c = *reinterpret_cast<const float2 *>(&Bs[b][k][tx * 2]);
+            acc[0][0] = fmaf(a.x, c.x, acc[0][0]); acc[0][1] = fmaf(a.x, c.y, acc[0][1]);
+            acc[1][0] = fmaf(a.y, c.x, acc[1][0]); acc[1][1] = fmaf(a.y, c.y, acc[1][1]);
+            acc[2][0] = fmaf(a.z, c.x, acc[2][0]); acc[2][1] = fmaf(a.z, c.y, acc[2][1]);
+            acc[3][0] = fmaf(a.w, c.x, acc[3][0]); acc[3][1] = fmaf(a.w, c.y, acc[3][1]);
+        }
+    }
+    float *dst = direct ? out : part + (int64_t)blockIdx.y * n * n;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int64_t gi = i0 + ty * 4 + i;
+        if (gi >= n) continue;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int64_t gj = j0 + tx * 2 + j;
+            if (gj >= n) continue;
+            if (direct) {
+                dst[gi * n + gj] += acc[i][j];
+                if (MODE == 0 && ti != tj) dst[gj * n + gi] += acc[i][j];
+            } else {
+                dst[gi * n + gj] = acc[i][j];
+                // (the reduction mirrors 128-wide blocks below the diagonal and
+                // reads diagonal ones in full)
+                if (MODE == 0 && ti != tj && gi / TB == gj / TB) dst[gj * n + gi] = acc[i][j];
+            }
+        }
+    }
+}
+
 // out[i][j] += sum_s part[s][i][j] in split order; mirrored for mode 0
 template <int MODE>
 __global__ void hess_reduce_kernel(int64_t n, int splits, const float *part, float *out) {
@@ -133,11 +227,24 @@ realq_status_t run(cudaStream_t s, int64_t n, int64_t T, const TX *X, const TX *
     float *partH = static_cast<float *>(ws);
     float *partD = partH + (size_t)splits * n * n;
     const int direct = splits == 1;
+    // 32 x 32 tiles while the 128 x 128 ones would leave SMs idle (both give
+    // the same bits)
+    const int nts = ceil_div(n, SB);
+    const bool vec = n % 4 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Xf)) & 15) == 0;
+    auto small = [&](auto mode, const TX *xf, float *o, float *p) {
+        constexpr int M = decltype(mode)::value;
+        const dim3 g((unsigned)(M == 0 ? (int64_t)nts * (nts + 1) / 2 : (int64_t)nts * nts), splits);
+        if (vec) hess_small_kernel<TX, M, true><<<g, STHREADS, 0, s>>>(n, T, X, xf, o, p, tper, direct);
+        else hess_small_kernel<TX, M, false><<<g, STHREADS, 0, s>>>(n, T, X, xf, o, p, tper, direct);
+    };
     if (H) {
         {
             Launch L("hessian_syrk_simt", s);
-            hess_kernel<TX, 0><<<dim3((unsigned)lower, splits), THREADS, 0, s>>>(n, T, X, nullptr, H, partH, tper,
-                                                                                 direct);
+            if (lower * splits < num_sms())
+                small(std::integral_constant<int, 0>(), nullptr, H, partH);
+            else
+                hess_kernel<TX, 0><<<dim3((unsigned)lower, splits), THREADS, 0, s>>>(n, T, X, nullptr, H, partH, tper,
+                                                                                     direct);
         }
         REALQ_TRY(check_launch("hessian_syrk_simt"));
         if (!direct) REALQ_TRY(hessian_reduce(s, n, splits, partH, H, 0));
@@ -145,7 +252,10 @@ realq_status_t run(cudaStream_t s, int64_t n, int64_t T, const TX *X, const TX *
     if (Xf) {
         {
             Launch L("hessian_cross_simt", s);
-            hess_kernel<TX, 1><<<dim3((unsigned)((int64_t)nt * nt), splits), THREADS, 0, s>>>(n, T, X, Xf, D, partD,
+            if ((int64_t)nt * nt * splits < num_sms())
+                small(std::integral_constant<int, 1>(), Xf, D, partD);
+            else
+                hess_kernel<TX, 1><<<dim3((unsigned)((int64_t)nt * nt), splits), THREADS, 0, s>>>(n, T, X, Xf, D, partD,
                                                                                              tper, direct);
         }
         REALQ_TRY(check_launch("hessian_cross_simt"));
