@@ -36,6 +36,8 @@
 #include "kernels.cuh"
 #include "tc.cuh"
 
+#include <type_traits>
+
 namespace realq {
 namespace {
 
@@ -1048,6 +1050,84 @@ namespace {
 // two s that puts it in [2^14, 2^15) (from its exponent field; clamped so
 // that s and 1/s are normal floats), then the fp16 planes of s v.  The
 // largest scaled value stays below 2^15 after rounding, within fp16's range.
+//
+// The row is held in registers between the two uses, NV float4 per thread, so
+// that each operand is read once (the pass is bound by memory: a 4096 x 4096
+// blend of F and F_next moves 201 MB instead of 335).
+// alpha x + (1 - alpha) y, rounded the same way wherever a blend is formed
+__device__ __forceinline__ float fblend(float alpha, float x, float y) {
+    return __fmaf_rn(alpha, x, __fmul_rn(1.f - alpha, y));
+}
+__device__ __forceinline__ float f16_row_scale(float mx, float *inv) {
+    // mx < 2^(e - 126) for biased exponent e: s = 2^(141 - e)
+    const int e = (int)((__float_as_uint(mx) >> 23) & 0xFFu);
+    int k = mx == 0.f ? 0 : 141 - e;
+    k = k < -126 ? -126 : (k > 126 ? 126 : k);
+    if (threadIdx.x == 0) *inv = __uint_as_float((uint32_t)(127 - k) << 23);
+    return __uint_as_float((uint32_t)(k + 127) << 23);
+}
+__device__ __forceinline__ float cta_max(float mx, float *red) {
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
+    __syncthreads();
+    mx = red[0];
+    for (int w = 1; w < 8; ++w) mx = fmaxf(mx, red[w]);
+    return mx;
+}
+
+// c0 .. c1 a multiple of 4 wide, at most 1024 NV; rows and planes 16- and 8-byte aligned
+template <int NV>
+__global__ void __launch_bounds__(256) split_f16_held_kernel(int64_t c0, int64_t c1, const float *x, const float *y,
+                                                             float alpha, int64_t lds, __half *hi, __half *lo,
+                                                             int64_t ldd, float *inv) {
+    __shared__ float red[8];
+    const int64_t r = blockIdx.x;
+    const float *xr = x + r * lds + c0;
+    const float *yr = y ? y + r * lds + c0 : nullptr;
+    const int w = (int)(c1 - c0);
+    float4 v[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        const int c = (i * 256 + threadIdx.x) * 4;
+        v[i] = c < w ? *reinterpret_cast<const float4 *>(xr + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    if (yr) {
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            const int c = (i * 256 + threadIdx.x) * 4;
+            if (c >= w) continue;
+            const float4 u = *reinterpret_cast<const float4 *>(yr + c);
+            v[i].x = fblend(alpha, v[i].x, u.x);
+            v[i].y = fblend(alpha, v[i].y, u.y);
+            v[i].z = fblend(alpha, v[i].z, u.z);
+            v[i].w = fblend(alpha, v[i].w, u.w);
+        }
+    }
+    float mx = 0.f;
+#pragma unroll
+    for (int i = 0; i < NV; ++i)
+        mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v[i].x), fabsf(v[i].y)), fmaxf(fabsf(v[i].z), fabsf(v[i].w))));
+    const float sc = f16_row_scale(cta_max(mx, red), inv + r);
+    __half *hr = hi + r * ldd + c0, *lr = lo + r * ldd + c0;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+        const int c = (i * 256 + threadIdx.x) * 4;
+        if (c >= w) continue;
+        const float f[4] = {v[i].x * sc, v[i].y * sc, v[i].z * sc, v[i].w * sc};
+        __half2 h[2], l[2];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const __half g = __float2half_rn(f[q]);
+            const __half d = __float2half_rn(f[q] - __half2float(g));
+            if (q & 1) h[q >> 1].y = g, l[q >> 1].y = d;
+            else h[q >> 1].x = g, l[q >> 1].x = d;
+        }
+        *reinterpret_cast<uint2 *>(hr + c) = *reinterpret_cast<const uint2 *>(h);
+        *reinterpret_cast<uint2 *>(lr + c) = *reinterpret_cast<const uint2 *>(l);
+    }
+}
+
+// rows wider than the registers hold: two passes over them
 __global__ void __launch_bounds__(256) split_f16_rows_kernel(int64_t c0, int64_t c1, const float *x, const float *y,
                                                              float alpha, int64_t lds, __half *hi, __half *lo,
                                                              int64_t ldd, float *inv) {
@@ -1057,23 +1137,13 @@ __global__ void __launch_bounds__(256) split_f16_rows_kernel(int64_t c0, int64_t
     const float *yr = y ? y + r * lds : nullptr;
     float mx = 0.f;
     for (int64_t c = c0 + threadIdx.x; c < c1; c += 256) {
-        const float v = yr ? alpha * xr[c] + (1.f - alpha) * yr[c] : xr[c];
+        const float v = yr ? fblend(alpha, xr[c], yr[c]) : xr[c];
         mx = fmaxf(mx, fabsf(v));
     }
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
-    __syncthreads();
-    mx = red[0];
-    for (int w = 1; w < 8; ++w) mx = fmaxf(mx, red[w]);
-    // mx < 2^(e - 126) for biased exponent e: s = 2^(141 - e)
-    const int e = (int)((__float_as_uint(mx) >> 23) & 0xFFu);
-    int k = mx == 0.f ? 0 : 141 - e;
-    k = k < -126 ? -126 : (k > 126 ? 126 : k);
-    const float sc = __uint_as_float((uint32_t)(k + 127) << 23);
-    if (threadIdx.x == 0) inv[r] = __uint_as_float((uint32_t)(127 - k) << 23);
+    const float sc = f16_row_scale(cta_max(mx, red), inv + r);
     __half *hr = hi + r * ldd, *lr = lo + r * ldd;
     for (int64_t c = c0 + threadIdx.x; c < c1; c += 256) {
-        const float v = (yr ? alpha * xr[c] + (1.f - alpha) * yr[c] : xr[c]) * sc;
+        const float v = (yr ? fblend(alpha, xr[c], yr[c]) : xr[c]) * sc;
         const __half h = __float2half_rn(v);
         hr[c] = h;
         lr[c] = __float2half_rn(v - __half2float(h));
@@ -1092,7 +1162,20 @@ realq_status_t tc_split_f16_rows(cudaStream_t s, int64_t rows, int64_t c0, int64
     if (rows > 0x7FFFFFFFll) return fail(REALQ_ERR_INVALID_ARG, "f16 split: too many rows");
     {
         Launch L("f16_split", s);
-        split_f16_rows_kernel<<<(unsigned)rows, 256, 0, s>>>(c0, c1, x, y, alpha, lds, hi, lo, ldd, inv);
+        const int64_t w = c1 - c0;
+        const uintptr_t al = reinterpret_cast<uintptr_t>(x + c0) | reinterpret_cast<uintptr_t>(y ? y + c0 : x + c0) |
+                             (reinterpret_cast<uintptr_t>(hi + c0) << 1) | (reinterpret_cast<uintptr_t>(lo + c0) << 1);
+        const bool held = w % 4 == 0 && lds % 4 == 0 && ldd % 4 == 0 && (al & 15) == 0 && w <= 16384;
+        auto go = [&](auto nv) {
+            split_f16_held_kernel<decltype(nv)::value><<<(unsigned)rows, 256, 0, s>>>(c0, c1, x, y, alpha, lds, hi, lo,
+                                                                                      ldd, inv);
+        };
+        if (!held) split_f16_rows_kernel<<<(unsigned)rows, 256, 0, s>>>(c0, c1, x, y, alpha, lds, hi, lo, ldd, inv);
+        else if (w <= 1024) go(std::integral_constant<int, 1>());
+        else if (w <= 2048) go(std::integral_constant<int, 2>());
+        else if (w <= 4096) go(std::integral_constant<int, 4>());
+        else if (w <= 8192) go(std::integral_constant<int, 8>());
+        else go(std::integral_constant<int, 16>());
     }
     return check_launch("f16_split");
 }
