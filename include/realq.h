@@ -496,12 +496,12 @@ void realq_graph_destroy(realq_graph_t graph);
 realq_status_t realq_set_tensor_tile(int mode);
 
 /* Tuning: the kernel of the column-serial quantize-and-compensate step.  0
- * (default): the kernel whose warps meet at a block-wide barrier after every
- * 32 columns; 1: warps pipelined through shared-memory progress flags where
- * the group parameters are taken at the block start or before it (more
- * instructions per warp for its polling and chunked updates: slower on
- * GB300, 41 against 31 us per 8192-row block).  Both perform the same
- * operations in the same order (identical results).
+ * (default): eight lanes per row, each holding every eighth column of the
+ * block, a row's columns one after another without a barrier; 1: a warp per 32
+ * columns with its lanes over the rows, the warps pipelined through
+ * shared-memory progress flags, where the group parameters are taken at the
+ * block start or before it (slower).  Both perform the same operations in the
+ * same order (identical results).
  * Process-wide.  REALQ_ERR_INVALID_ARG for other values.  No counterpart in
  * the paper. */
 realq_status_t realq_set_quant_kernel(int mode);

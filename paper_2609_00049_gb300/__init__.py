@@ -657,8 +657,8 @@ def realq_set_tensor_tile(mode: int) -> None:
 
 
 def realq_set_quant_kernel(mode: int) -> None:
-    """Kernel of the column-serial quantizer: 0 with block-wide barriers
-    (default), 1 pipelined (identical results)."""
+    """Kernel of the column-serial quantizer: 0 eight lanes per row (default),
+    1 pipelined warps (identical results)."""
     _check(lib().realq_set_quant_kernel(int(mode)))
 
 

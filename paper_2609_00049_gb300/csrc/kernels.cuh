@@ -85,9 +85,9 @@ void tc_set_tile_mode(int mode);
 // main loop; 2: the gradient-factor product too; 0: one tile per CTA
 // (process-wide).
 void tc_set_overlap(int mode);
-// The column-serial quantizer: 0 the barrier-phased kernel everywhere
-// (default), 1 the pipelined kernel where the group parameters come at the
-// block start or before it (process-wide).
+// The column-serial quantizer: 0 eight lanes per row (default), 1 the
+// pipelined kernel (a warp per 32 columns) where the group parameters come at
+// the block start or before it (process-wide).
 void quant_set_kernel(int mode);
 // hi / lo planes of the transpose of the rows x cols block at src (row stride
 // lds): dst[c * ldd + r] for r < rows, c < cols.

@@ -8,6 +8,7 @@
 #include "kernels.cuh"
 
 #include <cmath>
+#include <type_traits>
 
 namespace realq {
 namespace {
@@ -77,211 +78,286 @@ struct QArgs {
     float *Et;
     int64_t ldet;          // leading dimension of Et (all rows of the layer)
     int *status;
+    // the lazy update's planes out of the same launch (Eh null: Et instead);
+    // nq: CTAs of rows, the others transpose the U panel
+    float *Eh, *El, *Ph, *Pl;
+    int nq;
 };
 
-// Column-serial quantize + in-block OBS propagation for block [bs, bs + kb).
-// A CTA takes QB_ROWS rows and B/32 warps: warp w keeps columns
-// [32w, 32w + 32) of the CTA's rows in registers (lane = row).  Phase s: warp
-// s quantizes its 32 columns one after the other, feeding each column's error
-// to its later columns at once, and publishes the 32 errors of every row;
-// then every warp w > s applies them to its columns, column by column in
-// order, so each weight sees exactly the updates of the plain column loop.
-// U's B x B diagonal block is staged once in shared memory (rows padded to
-// keep float4 reads aligned).  G > 0: group parameters are computed at every
-// G-th column (a multiple of 32) from the current weights, with the min / max
-// of the group's sub-blocks gathered through shared memory; G = 0: they were
-// computed before the block.
-constexpr int QB_ROWS = 32;
+// Column-serial quantize + in-block OBS propagation for block [bs, bs + kb):
+// each column is quantized and its error fed to the later columns of the block
+// at once, so each weight sees the updates of the plain column loop in order.
+//
+// Eight lanes share a row (lane c holds columns 32 s + 4 c .. + 3), a warp four
+// rows, or eight with NR = 2, and a row never leaves its lanes: the owner's
+// weight goes to the other seven by a shuffle, all eight form the code and the
+// error, and each updates its own later columns.  No barrier orders the columns
+// (warps that owned 32 columns each met at one after every 32), and the loop
+// over the lanes stays rolled, so that the code runs from the instruction cache
+// instead of streaming through it once per block.  What bounds it is the chain
+// from one column to the next (shuffle, product, rounding, clamp, error,
+// update) and about 40 instructions per column and warp.  A 128-column block of
+// 1024 rows: 28 -> 13 us, and the 4 us launch that made the lazy update's planes
+// is gone.
+//
+// U's B x B diagonal block is copied to shared memory row group by row group
+// (32 rows each) ahead of the columns that read it.  G > 0: group parameters are
+// computed at every G-th column (a multiple of 32) from the current weights; G =
+// 0: they were computed before the block.
+//
+// PL: the operands of the lazy batch update on the tensor cores come out of the
+// same launch: the errors as K-major tf32 planes of -E (rows of E as they are),
+// and the CTAs from nq on transpose the block's U panel into its planes (they
+// depend on U alone and run beside the rows).
+constexpr int QB_ROWS = 32;       // rows per CTA of the pipelined variant below
 }  // namespace
 constexpr int kGSplit = 8;   // K slices of the next block's G product
 namespace {
 
-template <int B, int G>
-__global__ void __launch_bounds__(B) quant_block_kernel(const QArgs a) {
-    constexpr int NW = B / 32;            // warps = sub-blocks
-    constexpr int UP = B + 4;             // U row pitch (floats)
+__device__ __forceinline__ void cp16(float *dst, const float *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ float tf32_top(float x) { return __int_as_float(__float_as_int(x) & (int)0xFFFFE000u); }
+
+constexpr int QT = 128;           // threads per CTA: 4 warps
+
+template <int B, int G, int NR, bool PL>
+__global__ void __launch_bounds__(QT) quant_rows_kernel(const QArgs a) {
+    constexpr int NS = B / 32;                 // sub-blocks of 32 columns
     extern __shared__ __align__(16) float qsm[];
-    float *Us = qsm;                      // B x UP: U[j][k] for j < k, else 0
-    float *invd = Us + B * UP;            // B
-    float *Es = invd + B;                 // QB_ROWS x 33: errors of the current sub-block
-    float *mm = Es + QB_ROWS * 33;        // 2 x NW x QB_ROWS: group min / max partials
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float *Us = qsm;                           // B x B: row j of U's diagonal block
+    float *invd = Us + B * B;                  // B
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cl = lane & 7;
     const int kb = a.kb;
-    if ((a.n & 3) == 0 && kb == B) {
-        // (unrolled so that several loads are in flight per thread)
-#pragma unroll 8
-        for (int idx = threadIdx.x; idx < B * B / 4; idx += blockDim.x) {
-            const int j = (idx * 4) / B, k = (idx * 4) % B;
-            const float4 v = *reinterpret_cast<const float4 *>(a.U + (a.bs + j) * a.n + a.bs + k);
-            float *d = Us + j * UP + k;
-            d[0] = (k + 0 > j) ? v.x : 0.f;
-            d[1] = (k + 1 > j) ? v.y : 0.f;
-            d[2] = (k + 2 > j) ? v.z : 0.f;
-            d[3] = (k + 3 > j) ? v.w : 0.f;
-        }
-    } else {
-        for (int idx = threadIdx.x; idx < B * B; idx += blockDim.x) {
-            const int j = idx / B, k = idx % B;
-            Us[j * UP + k] = (j < kb && k < kb && k > j) ? a.U[(a.bs + j) * a.n + a.bs + k] : 0.f;
-        }
-    }
-    for (int j = threadIdx.x; j < B; j += blockDim.x)
-        invd[j] = (j < kb) ? 1.f / a.U[(a.bs + j) * a.n + a.bs + j] : 0.f;
-
-    const int64_t i = (int64_t)blockIdx.x * QB_ROWS + lane;   // this lane's row
-    const bool live = i < a.m;
-    const int c0 = warp * 32;                                   // this warp's first column
-    float r[32];
-    {
-        const float *wrow = a.W + (live ? i : 0) * a.n + a.bs + c0;
-        if ((a.n & 3) == 0 && c0 + 32 <= kb) {
+    if (PL && (int)blockIdx.x >= a.nq) {
+        // a 32 x 32 tile of the U panel: P[j][k] = U[bs + k][be + j], hi and lo
+        float(*tile)[33] = reinterpret_cast<float(*)[33]>(qsm);
+        const int64_t t = blockIdx.x - a.nq;
+        const int64_t be = a.bs + B, rcols = a.n - be;
+        const int64_t tj = t / (B / 32);
+        const int tk = (int)(t % (B / 32));
+        const int64_t j = tj * 32 + lane;
 #pragma unroll
-            for (int c = 0; c < 32; c += 4) {
-                const float4 v = live ? *reinterpret_cast<const float4 *>(wrow + c) : make_float4(0.f, 0.f, 0.f, 0.f);
-                r[c] = v.x; r[c + 1] = v.y; r[c + 2] = v.z; r[c + 3] = v.w;
+        for (int q = warp; q < 32; q += QT / 32)
+            tile[q][lane] = j < rcols ? a.U[(a.bs + tk * 32 + q) * a.n + be + j] : 0.f;
+        __syncthreads();
+#pragma unroll
+        for (int q = warp; q < 32; q += QT / 32) {
+            const int64_t c = tj * 32 + q;
+            if (c < rcols) {
+                const float v = tile[lane][q], h = tf32_top(v);
+                a.Ph[c * B + tk * 32 + lane] = h;
+                a.Pl[c * B + tk * 32 + lane] = v - h;
+            }
+        }
+        return;
+    }
+    const bool vec = (a.n & 3) == 0 && (reinterpret_cast<uintptr_t>(a.U) & 15) == 0 && kb == B;
+    for (int s = 0; s < B / 32; ++s) {
+        // rows 32 s .. of the block, from column 32 s on (the earlier ones are never read)
+        if (vec) {
+            const int w4 = (B - 32 * s) / 4;
+            for (int idx = threadIdx.x; idx < 32 * w4; idx += QT) {
+                const int j = 32 * s + idx / w4, k = 32 * s + (idx % w4) * 4;
+                cp16(Us + j * B + k, a.U + (a.bs + j) * a.n + a.bs + k);
             }
         } else {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) r[c] = (live && c0 + c < kb) ? wrow[c] : 0.f;
+            for (int idx = threadIdx.x; idx < 32 * B; idx += QT) {
+                const int j = 32 * s + idx / B, k = idx % B;
+                Us[j * B + k] = (j < kb && k < kb) ? a.U[(a.bs + j) * a.n + a.bs + k] : 0.f;
+            }
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");
     }
-    float sc = 1.f, zr = 0.f;
-    if (G == 0 && live) {
-        const int gi = (int)(a.bs / a.g);
-        sc = a.scale[i * a.ngroups + gi];
-        zr = (float)a.zero[i * a.ngroups + gi];
-    }
-    __syncthreads();
+    for (int j = threadIdx.x; j < B; j += QT) invd[j] = (j < kb) ? 1.f / a.U[(a.bs + j) * a.n + a.bs + j] : 0.f;
 
+    int64_t row[NR];
+    bool live[NR];
+    float w[NR][NS][4], sc[NR], zr[NR], rcp[NR];
+    // the scale's reciprocal and the products with it stay normal numbers
+    bool plain = true;
+    auto recip = [&](int x) {
+        rcp[x] = __frcp_rn(sc[x]);
+        if (!(sc[x] > 1e-30f && sc[x] < 1e30f)) plain = false;
+    };
+    const bool wvec = (a.n & 3) == 0 && kb == B && (reinterpret_cast<uintptr_t>(a.W) & 15) == 0;
+#pragma unroll
+    for (int x = 0; x < NR; ++x) {
+        row[x] = ((int64_t)blockIdx.x * (QT / 32) + warp) * (4 * NR) + 4 * x + (lane >> 3);
+        live[x] = row[x] < a.m;
+        const float *wr = a.W + (live[x] ? row[x] : 0) * a.n + a.bs + 4 * cl;
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            if (wvec) {
+                const float4 v = live[x] ? *reinterpret_cast<const float4 *>(wr + 32 * s) : make_float4(0.f, 0.f, 0.f, 0.f);
+                w[x][s][0] = v.x; w[x][s][1] = v.y; w[x][s][2] = v.z; w[x][s][3] = v.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) w[x][s][e] = (live[x] && 32 * s + 4 * cl + e < kb) ? wr[32 * s + e] : 0.f;
+            }
+        }
+        sc[x] = 1.f;
+        zr[x] = 0.f;
+        if (G == 0 && live[x]) {
+            const int gi = (int)(a.bs / a.g);
+            sc[x] = a.scale[row[x] * a.ngroups + gi];
+            zr[x] = (float)a.zero[row[x] * a.ngroups + gi];
+        }
+        recip(x);
+    }
     const float maxq = (float)((1 << a.bits) - 1);
-    bool bad = false;
-#pragma unroll 1
-    for (int s = 0; s < NW && s * 32 < kb; ++s) {
-        if (G > 0 && ((s * 32) % (G > 0 ? G : 1)) == 0) {
-            // min / max of the group's columns (sub-blocks s .. s + G/32 - 1)
+    float poison = 0.f;            // NaN once a non-finite weight was met
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        // U's rows of these 32 columns have landed
+        if (s == 0) asm volatile("cp.async.wait_group %0;" ::"n"(NS - 1) : "memory");
+        else if (s == 1) asm volatile("cp.async.wait_group %0;" ::"n"(NS > 1 ? NS - 2 : 0) : "memory");
+        else if (s == 2) asm volatile("cp.async.wait_group %0;" ::"n"(NS > 2 ? NS - 3 : 0) : "memory");
+        else asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (32 * s >= kb) continue;
+        if (G > 0 && (32 * s) % (G > 0 ? G : 1) == 0) {
             constexpr int GS = (G > 0 ? G : 32) / 32;
-            if (warp >= s && warp < s + GS) {
+#pragma unroll
+            for (int x = 0; x < NR; ++x) {
                 float mn = 0.f, mx = 0.f;
 #pragma unroll
-                for (int c = 0; c < 32; ++c)
-                    if (c0 + c < kb) {
-                        mn = fminf(mn, r[c]);
-                        mx = fmaxf(mx, r[c]);
-                    }
-                mm[warp * QB_ROWS + lane] = mn;
-                mm[(NW + warp) * QB_ROWS + lane] = mx;
-            }
-            __syncthreads();
-            if (warp == s) {
-                float mn = 0.f, mx = 0.f;
-                for (int w = s; w < s + GS && w < NW; ++w) {
-                    mn = fminf(mn, mm[w * QB_ROWS + lane]);
-                    mx = fmaxf(mx, mm[(NW + w) * QB_ROWS + lane]);
+                for (int q = s; q < s + GS && q < NS; ++q)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        if (PL || 32 * q + 4 * cl + e < kb) {
+                            mn = fminf(mn, w[x][q][e]);
+                            mx = fmaxf(mx, w[x][q][e]);
+                        }
+#pragma unroll
+                for (int o = 4; o > 0; o >>= 1) {
+                    mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
                 }
-                grid_params(mn, mx, a.bits, a.sym, sc, zr);
-                if (live) {
-                    const int gi = (int)((a.bs + s * 32) / a.g);
-                    a.scale[i * a.ngroups + gi] = sc;
-                    a.zero[i * a.ngroups + gi] = (uint8_t)zr;
+                grid_params(mn, mx, a.bits, a.sym, sc[x], zr[x]);
+                if (live[x] && cl == 0) {
+                    const int gi = (int)((a.bs + 32 * s) / a.g);
+                    a.scale[row[x] * a.ngroups + gi] = sc[x];
+                    a.zero[row[x] * a.ngroups + gi] = (uint8_t)zr[x];
                 }
-                // the next sub-blocks of the same group quantize with these parameters
-                mm[lane] = sc;
-                mm[QB_ROWS + lane] = zr;
-            }
-            __syncthreads();
-            if (warp > s && warp < s + GS) {
-                sc = mm[lane];
-                zr = mm[QB_ROWS + lane];
+                recip(x);
             }
         }
-        if (warp == s) {
-            uint32_t packed[4] = {0u, 0u, 0u, 0u};
-            // rint(w / sc) through the reciprocal: x = w * rn(1/sc) is within
-            // 3 * 2^-24 |w / sc| of the quotient and of its IEEE rounding, so
-            // where x is farther than 4 * 2^-24 |x| from every half-integer
-            // both round to the same integer; nearer (and for non-finite
-            // values) the IEEE division decides, so the code is the one of
-            // rint(w / sc) in every case and the chain from one column's
-            // error to the next column's code avoids the division
-            const float rcp = __frcp_rn(sc);
-#pragma unroll
-            for (int jj = 0; jj < 32; ++jj) {
-                const int j = c0 + jj;
-                float err = 0.f;
-                uint32_t qi = 0;
-                if (j < kb) {
-                    const float w = r[jj];
-                    bad |= !isfinite(w);
-                    const float x = __fmul_rn(w, rcp);
-                    float qx = rintf(x);
-                    const float gap = 0.5f - fabsf(x - qx);
-                    if (!(gap > 2.4e-7f * fabsf(x) + 1e-30f)) qx = rintf(w / sc);
-                    float q = qx + zr;
-                    q = fminf(fmaxf(q, 0.f), maxq);
-                    const float dq = sc * (q - zr);
-                    err = (w - dq) * invd[j];
-                    r[jj] = dq;
-                    qi = (uint32_t)q;
-#pragma unroll
-                    for (int kk = jj + 1; kk < 32; ++kk) r[kk] = fmaf(-err, Us[j * UP + c0 + kk], r[kk]);
-                }
-                Es[lane * 33 + jj] = err;
-                if (live && j < kb) a.Et[(int64_t)j * a.ldet + i] = err;
-                packed[jj >> 3] |= (qi & 15u) << ((jj & 7) * 4);
-            }
-            if (live) {
-                uint8_t *crow = a.codes + i * a.ncb + (a.bs + c0) / 2;
-                if (c0 + 32 <= kb && (((uintptr_t)crow) & 15) == 0) {
-                    *reinterpret_cast<uint4 *>(crow) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                } else {
-                    for (int jj = 0; jj < 32 && c0 + jj < kb; jj += 2)
-                        crow[jj / 2] = (uint8_t)((packed[jj >> 3] >> ((jj & 7) * 4)) & 0xFFu);
-                }
-            }
-        }
-        __syncthreads();
-        if (warp > s) {
-            // the 32 errors of sub-block s, column by column in order (the
-            // column loop stays rolled: the kernel's code then fits the
-            // instruction cache)
+        // the errors and codes (as floats) of this lane's four columns
+        float er[NR][4] = {}, qf[NR][4] = {};
+        const int cmax = PL ? 8 : min(8, (kb - 32 * s + 3) / 4);
+        // rint(v / sc) without a division or a branch: t = v rn(1 / sc) is
+        // within two units in the last place of the quotient, and t + (v - t sc)
+        // rn(1 / sc) rounds to the IEEE quotient (Markstein's theorem: the
+        // remainder by FMA, the reciprocal correctly rounded); adding and taking
+        // away 1.5 * 2^23 rounds that to the nearest even integer.  (The clamp
+        // first: a quotient beyond +-64 ends at the same end of the grid, and
+        // infinities stay clear of inf - inf.)  Scales outside 1e-30 .. 1e30
+        // take the division.
+        auto columns = [&](auto exact) {
 #pragma unroll 1
-            for (int jj = 0; jj < 32; ++jj) {
-                const float ej = Es[lane * 33 + jj];
-                const float *urow = Us + (s * 32 + jj) * UP + c0;
+            for (int c = 0; c < cmax; ++c) {
+                const int j0 = 32 * s + 4 * c;
+                const bool own = cl == c, after = cl > c;
+                const float4 id4 = *reinterpret_cast<const float4 *>(invd + j0);
+                const float idv[4] = {id4.x, id4.y, id4.z, id4.w};
 #pragma unroll
-                for (int c = 0; c < 32; c += 4) {
-                    const float4 u = *reinterpret_cast<const float4 *>(urow + c);
-                    r[c] = fmaf(-ej, u.x, r[c]);
-                    r[c + 1] = fmaf(-ej, u.y, r[c + 1]);
-                    r[c + 2] = fmaf(-ej, u.z, r[c + 2]);
-                    r[c + 3] = fmaf(-ej, u.w, r[c + 3]);
+                for (int e = 0; e < 4; ++e) {
+                    if (!PL && j0 + e >= kb) break;
+                    float4 uv[NS];
+#pragma unroll
+                    for (int q = s; q < NS; ++q)
+                        uv[q] = *reinterpret_cast<const float4 *>(Us + (j0 + e) * B + 32 * q + 4 * cl);
+#pragma unroll
+                    for (int x = 0; x < NR; ++x) {
+                        const float v = __shfl_sync(0xffffffffu, w[x][s][e], (lane & 24) | c);
+                        poison = fmaf(v, 0.f, poison);
+                        float q;
+                        if (decltype(exact)::value) {
+                            q = rintf(__fdiv_rn(v, sc[x]));
+                        } else {
+                            float t = fminf(fmaxf(__fmul_rn(v, rcp[x]), -64.f), 64.f);
+                            t = __fmaf_rn(__fmaf_rn(-t, sc[x], v), rcp[x], t);
+                            q = __fsub_rn(__fadd_rn(t, 12582912.f), 12582912.f);
+                        }
+                        q = fminf(fmaxf(__fadd_rn(q, zr[x]), 0.f), maxq);
+                        // (spelled out so that one row and two take the same roundings)
+                        const float qz = __fsub_rn(q, zr[x]), dq = __fmul_rn(sc[x], qz);
+                        const float err = __fmul_rn(__fsub_rn(v, dq), idv[e]), ne = -err;
+                        er[x][e] = own ? err : er[x][e];
+                        qf[x][e] = own ? q : qf[x][e];
+                        // the same sub-block: this lane's columns past j0 + e
+                        const float us[4] = {uv[s].x, uv[s].y, uv[s].z, uv[s].w};
+#pragma unroll
+                        for (int f = 0; f < 4; ++f) {
+                            const float up = __fmaf_rn(ne, us[f], w[x][s][f]);
+                            if (f == e) w[x][s][f] = own ? dq : (after ? up : w[x][s][f]);
+                            else w[x][s][f] = (after || (own && f > e)) ? up : w[x][s][f];
+                        }
+                        // the later ones
+#pragma unroll
+                        for (int k = s + 1; k < NS; ++k) {
+                            w[x][k][0] = __fmaf_rn(ne, uv[k].x, w[x][k][0]);
+                            w[x][k][1] = __fmaf_rn(ne, uv[k].y, w[x][k][1]);
+                            w[x][k][2] = __fmaf_rn(ne, uv[k].z, w[x][k][2]);
+                            w[x][k][3] = __fmaf_rn(ne, uv[k].w, w[x][k][3]);
+                        }
+                    }
                 }
             }
-        }
-        __syncthreads();
-    }
-    if (live) {
-        float *wout = a.W + i * a.n + a.bs + c0;
-        if ((a.n & 3) == 0 && c0 + 32 <= kb) {
+        };
+        if (__all_sync(0xffffffffu, plain)) columns(std::false_type());
+        else columns(std::true_type());
+        // these 32 columns are final: weights, errors, codes
 #pragma unroll
-            for (int c = 0; c < 32; c += 4) *reinterpret_cast<float4 *>(wout + c) = make_float4(r[c], r[c + 1], r[c + 2], r[c + 3]);
-        } else {
+        for (int x = 0; x < NR; ++x) {
+            if (!live[x]) continue;
+            const int j0 = 32 * s + 4 * cl;
+            float *wo = a.W + row[x] * a.n + a.bs + j0;
+            uint32_t word = 0;
 #pragma unroll
-            for (int c = 0; c < 32; ++c)
-                if (c0 + c < kb) wout[c] = r[c];
+            for (int e = 0; e < 4; ++e) word |= ((uint32_t)qf[x][e] & 15u) << (4 * e);
+            uint8_t *crow = a.codes + row[x] * a.ncb + (a.bs + j0) / 2;
+            if (wvec) {
+                *reinterpret_cast<float4 *>(wo) = make_float4(w[x][s][0], w[x][s][1], w[x][s][2], w[x][s][3]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (j0 + e < kb) wo[e] = w[x][s][e];
+            }
+            if (j0 + 3 < kb && (reinterpret_cast<uintptr_t>(crow) & 1) == 0) {
+                *reinterpret_cast<uint16_t *>(crow) = (uint16_t)word;
+            } else {
+                if (j0 < kb) crow[0] = (uint8_t)word;
+                if (j0 + 2 < kb) crow[1] = (uint8_t)(word >> 8);
+            }
+            if (PL) {
+                float h[4], l[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    h[e] = tf32_top(-er[x][e]);
+                    l[e] = -er[x][e] - h[e];
+                }
+                *reinterpret_cast<float4 *>(a.Eh + row[x] * B + j0) = make_float4(h[0], h[1], h[2], h[3]);
+                *reinterpret_cast<float4 *>(a.El + row[x] * B + j0) = make_float4(l[0], l[1], l[2], l[3]);
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (j0 + e < kb) a.Et[(int64_t)(j0 + e) * a.ldet + row[x]] = er[x][e];
+            }
         }
     }
-    if (bad) atomicOr(a.status, ST_NONFINITE);
+    if (poison != 0.f) atomicOr(a.status, ST_NONFINITE);   // (NaN compares unequal)
 }
 
-// The same column-serial quantize + in-block OBS as quant_block_kernel, with
-// the phases pipelined: warp w applies sub-block s's errors in chunks of 8
+// The same column-serial quantize + in-block OBS with a warp per 32 columns, its
+// lanes the rows, and the warps pipelined: warp w applies sub-block s's errors in chunks of 8
 // columns as soon as warp s has published them (a per-warp progress flag in
 // shared memory) and starts its own chain right after, instead of every warp
 // waiting at a CTA barrier for the slowest one after every phase.  Each
 // weight still receives exactly the updates of the plain column loop in the
-// same order (sub-blocks in order, columns in order), so the results are the
-// kernel's above bit for bit.  U's diagonal block is staged as its 32 x 32
+// same order, so the results are the kernel's above bit for bit.  U's diagonal block is staged as its 32 x 32
 // blocks on or above the diagonal only (row pitch 36 keeps float4 reads
 // aligned), which leaves room for three CTAs per SM beside the error
 // buffers.  Group parameters at the block start (G = B) or before it (G = 0).
@@ -438,7 +514,7 @@ __global__ void __launch_bounds__(B) quant_block_pipe_kernel(const QArgs a) {
         float *Eo = Es + (warp < QP::NBUF ? warp : 0) * QB_ROWS * 33;
         const float *ud = Ut + qslot(warp, warp, NW) * 32 * P;
         uint32_t packed[4] = {0u, 0u, 0u, 0u};
-        // rint(w / sc) through the reciprocal, as in quant_block_kernel
+        // rint(w / sc) through the reciprocal, as in quant_rows_kernel
         const float rcp = __frcp_rn(sc);
 #pragma unroll
         for (int jj = 0; jj < 32; ++jj) {
@@ -588,18 +664,30 @@ __global__ void dot_final_kernel(const double *part, int nparts, float *out) {
 
 inline unsigned blocks_for(int64_t count, int threads = 256) { return (unsigned)((count + threads - 1) / threads); }
 
-template <int B, int G>
-realq_status_t launch_qb(cudaStream_t s, const QArgs &qa) {
-    const size_t smem = (size_t)(B * (B + 4) + B + QB_ROWS * 33 + 2 * (B / 32) * QB_ROWS) * sizeof(float);
-    REALQ_TRY(set_smem_limit(reinterpret_cast<const void *>(quant_block_kernel<B, G>), (int)smem));
+template <int B, int G, int NR, bool PL>
+realq_status_t launch_rows(cudaStream_t s, QArgs qa) {
+    const size_t smem = (size_t)(B * B + B) * sizeof(float);
+    REALQ_TRY(set_smem_limit(reinterpret_cast<const void *>(quant_rows_kernel<B, G, NR, PL>), (int)smem));
+    qa.nq = ceil_div(qa.m, QT / 32 * 4 * NR);
+    const int64_t panel = PL ? (int64_t)ceil_div(qa.n - qa.bs - B, 32) * (B / 32) : 0;
     {
         Launch L("quant_block", s);
-        quant_block_kernel<B, G><<<ceil_div(qa.m, QB_ROWS), B, smem, s>>>(qa);
+        quant_rows_kernel<B, G, NR, PL><<<(unsigned)(qa.nq + panel), QT, smem, s>>>(qa);
     }
     return check_launch("quant_block");
 }
 
-int g_quant_kernel = 0;   // 0: the barrier-phased quantizer (default), 1: the pipelined one where it applies
+// Rows per warp: four up to two CTAs of 16 rows per SM, then eight, which share
+// U's reads (a 128-column block: 13 us at 1024 rows with four; 18.5 us at 4096
+// to 9728 rows with eight, where four would need a second wave of CTAs).
+template <int B, int G>
+realq_status_t launch_qb(cudaStream_t s, const QArgs &qa) {
+    const bool two = qa.m > 32 * (int64_t)num_sms();
+    if (qa.Eh) return two ? launch_rows<B, G, 2, true>(s, qa) : launch_rows<B, G, 1, true>(s, qa);
+    return two ? launch_rows<B, G, 2, false>(s, qa) : launch_rows<B, G, 1, false>(s, qa);
+}
+
+int g_quant_kernel = 0;   // 0: eight lanes per row (default), 1: the pipelined warps where they apply
 }  // namespace
 
 void quant_set_kernel(int mode) { g_quant_kernel = mode; }
@@ -619,8 +707,9 @@ realq_status_t launch_qb_pipe(cudaStream_t s, const QArgs &qa) {
 
 template <int B>
 realq_status_t launch_qb_g(cudaStream_t s, const QArgs &qa, int Gk) {
-    if (g_quant_kernel == 1 && Gk == 0) return launch_qb_pipe<B, 0>(s, qa);
-    if (g_quant_kernel == 1 && Gk == B) return launch_qb_pipe<B, B>(s, qa);
+    // (the pipelined kernel writes E^T: the caller leaves Eh null for it)
+    if (g_quant_kernel == 1 && !qa.Eh && Gk == 0) return launch_qb_pipe<B, 0>(s, qa);
+    if (g_quant_kernel == 1 && !qa.Eh && Gk == B) return launch_qb_pipe<B, B>(s, qa);
     if (Gk == 0) return launch_qb<B, 0>(s, qa);
     if (Gk == B) return launch_qb<B, B>(s, qa);
     if (B >= 64 && Gk == B / 2) return launch_qb<B, (B >= 64 ? B / 2 : B)>(s, qa);
@@ -1161,6 +1250,9 @@ realq_status_t sweep_block(cudaStream_t s, SweepPlan &p, int64_t b) {
     }
     if (!params_here) REALQ_TRY(check_launch("group_params"));
     const int Gk = !params_here ? 0 : (p.group >= p.n ? B : p.group);
+    // one row group with the lazy update on the tensor cores: the quantizer
+    // writes that update's operands itself
+    const bool planes_here = p.trail_tc && p.rgroups == 1 && be < p.n && g_quant_kernel == 0;
     for (int gr = 0; gr < p.rgroups; ++gr) {
         // row group gr against its own U (one group: all rows, U)
         const int64_t row0 = gr * p.rg_rows, rows = std::min<int64_t>(p.rg_rows, p.m - row0);
@@ -1173,6 +1265,9 @@ realq_status_t sweep_block(cudaStream_t s, SweepPlan &p, int64_t b) {
         qa.scale = p.scale + row0 * p.ngroups; qa.zero = p.zero + row0 * p.ngroups; qa.codes = p.codes + row0 * ncb;
         qa.ncb = ncb;
         qa.Et = p.Et + row0; qa.ldet = p.m; qa.status = p.status;
+        if (planes_here) {
+            qa.Eh = p.Eh; qa.El = p.El; qa.Ph = p.UPh; qa.Pl = p.UPl;
+        }
         if (B == 128) REALQ_TRY(launch_qb_g<128>(s, qa, Gk));
         else if (B == 64) REALQ_TRY(launch_qb_g<64>(s, qa, Gk));
         else REALQ_TRY(launch_qb_g<32>(s, qa, Gk));
@@ -1199,8 +1294,9 @@ realq_status_t sweep_block(cudaStream_t s, SweepPlan &p, int64_t b) {
         for (int gr = 0; gr < p.rgroups; ++gr) {
             const int64_t row0 = gr * p.rg_rows, rows = std::min<int64_t>(p.rg_rows, p.m - row0);
             if (rows <= 0) break;
-            REALQ_TRY(tc_trail_planes(s, p.m, gr == 0 ? p.Et : nullptr, p.m, p.n, p.Ug + (size_t)gr * p.n * p.n, bs,
-                                      be, kb, B, p.Eh, p.El, p.UPh, p.UPl));
+            if (!planes_here)
+                REALQ_TRY(tc_trail_planes(s, p.m, gr == 0 ? p.Et : nullptr, p.m, p.n, p.Ug + (size_t)gr * p.n * p.n,
+                                          bs, be, kb, B, p.Eh, p.El, p.UPh, p.UPl));
             TcEpi e{};
             e.mode = TC_ACCUM;
             e.M = p.W + row0 * p.n;
