@@ -174,17 +174,15 @@ __device__ __forceinline__ void bgd_pg_rows4(const TcEpi &e, int64_t gi0, int64_
     }
 }
 
-// TC_ACCUM for 4 rows x 4 columns: M += acc
-__device__ __forceinline__ void accum_rows4(const TcEpi &e, int64_t gi0, int64_t gj, const float *t, int tp) {
+// TC_ACCUM for 4 rows x 4 columns: M = old + acc
+__device__ __forceinline__ void accum_rows4(const TcEpi &e, int64_t gi0, int64_t gj, const float *t, int tp,
+                                            const float4 (&old)[4]) {
     const int64_t col = e.col0 + gj;
-    float4 mp[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) mp[u] = ld4(e.M + (gi0 + u) * e.ldw + col);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const float *tr = t + u * tp;
         st4(e.M + (gi0 + u) * e.ldw + col,
-            make_float4(mp[u].x + tr[0], mp[u].y + tr[1], mp[u].z + tr[2], mp[u].w + tr[3]));
+            make_float4(old[u].x + tr[0], old[u].y + tr[1], old[u].z + tr[2], old[u].w + tr[3]));
     }
 }
 
@@ -329,6 +327,24 @@ __global__ void __launch_bounds__(THREADS, 1)
     tc::fence_after_sync();
     const uint32_t tmem = *tslot;
 
+    // TC_ACCUM: the output's old values are read while the operands arrive (a
+    // short product's epilogue is otherwise one round trip to memory per four
+    // rows: 4 of the lazy update's 13 to 19 us).  Batch b of this warp: rows
+    // warp RPW + 4 (b % (RPW / 4)) .., columns 128 (b / (RPW / 4)) + 4 lane ..
+    constexpr int RPW = TB / (THREADS / 32);   // tile rows per warp
+    constexpr int NBATCH = MODE == TC_ACCUM ? RPW / 4 * (TN / 128) : 1;
+    float4 old[NBATCH][4];
+    if (MODE == TC_ACCUM) {
+#pragma unroll
+        for (int b = 0; b < NBATCH; ++b) {
+            const int64_t gi = i0 + warp * RPW + 4 * (b % (RPW / 4)), gj = j0 + 128 * (b / (RPW / 4)) + lane * 4;
+            if (gi + 3 < M && gj + 3 < N) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) old[b][u] = ld4(e.M + (gi + u) * e.ldw + e.col0 + gj);
+            }
+        }
+    }
+
     if (warp == 0 && lane == 0) {
         // ---------------- TMA producer ----------------
         int it = 0;
@@ -432,13 +448,14 @@ __global__ void __launch_bounds__(THREADS, 1)
         // rows of the tile, each lane on 4 consecutive columns of a 128-wide
         // column half; the loads of 4 rows are issued before any store so
         // they overlap
-        constexpr int RPW = TB / (THREADS / 32);   // tile rows per warp
-#pragma unroll 1
+#pragma unroll (MODE == TC_ACCUM ? TN / 128 : 1)
         for (int ch = 0; ch < TN; ch += 128) {
             const int cc = ch + lane * 4;
             const int64_t gj = j0 + cc;
             const bool vec = MODE != TC_STORE && gj + 3 < N;
-            for (int rb = warp * RPW; rb < warp * RPW + RPW; rb += 4) {
+#pragma unroll (MODE == TC_ACCUM ? RPW / 4 : 1)
+            for (int rq = 0; rq < RPW; rq += 4) {
+                const int rb = warp * RPW + rq;
                 if (i0 + rb >= M) break;
                 // a batch of 4 rows runs vectorized when all 4 exist (M need
                 // not be a multiple of 4 for a row group)
@@ -446,7 +463,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     if (MODE == TC_ADAM) adam_rows4(e, i0 + rb, M, gj, T + rb * TP + cc, TP);
                     else if (MODE == TC_BGD_P) bgd_p_rows4(e, i0 + rb, M, gj, T + rb * TP + cc, TP);
                     else if (MODE == TC_BGD_PG) bgd_pg_rows4(e, i0 + rb, gj, T + rb * TP + cc, TP);
-                    else accum_rows4(e, i0 + rb, gj, T + rb * TP + cc, TP);
+                    else accum_rows4(e, i0 + rb, gj, T + rb * TP + cc, TP, old[(MODE == TC_ACCUM ? ch / 128 * (RPW / 4) + rq / 4 : 0)]);
                 } else {
                     for (int u = 0; u < 4; ++u) {
                         const int rr = rb + u;
