@@ -386,8 +386,9 @@ def work_models(wl, args=None):
             bgd_g += 2 * m * m * r
             trail += 2 * m * (be - b * B) * r
             if r > 0:
-                # the update's operands as tf32 planes: read E_b and the U
-                # panel once, write both planes of each
+                # the update's operands as tf32 planes where a pass of its own
+                # makes them (row groups; otherwise the quantizer writes them):
+                # read E_b and the U panel once, write both planes of each
                 trail_planes += 12 * (be - b * B) * (m + r)
             serial_bytes += m * (be - b * B) * (4 + 4 + 4) + m * (be - b * B) // 2
     if getattr(args, "a_loss_clip", None) and getattr(args, "minibatch_seqs", 0):
@@ -432,16 +433,17 @@ def work_models(wl, args=None):
     per_step["trailing_update"] = ("tf32x3", trail, "TFLOP/s")
     per_step["trailing_planes"] = ("hbm", trail_planes, "GB/s")
     per_step["quant_block"] = ("hbm", serial_bytes, "GB/s")
-    prep_flops = sum(2 * s.n ** 3 // 3 for s in wl.inputs.values())
     per_step["chol_diag"] = ("alu", sum(s.n * 64 * 64 for s in wl.inputs.values()), "TFLOP/s")
-    # the rank-64 updates: the look-ahead column on fp32 tiles (2 k0 64^2 flop
-    # per step, about 64 n^2 in all), the rest on the tensor cores; the
-    # triangular inverse's product on the tensor cores, or on fp32 tiles
-    # where the workspace lacks the planes of U^T
+    # the preparation of wide inputs: diagonal blocks of 512 columns by one
+    # cluster each (fp32 FFMA), the depth-512 updates and the rows of U on the
+    # tensor cores; the 64-wide steps (chol_diag, chol_update, trtri_trmm*) are
+    # those of a workspace without planes and of recorded profiles
+    per_step["chol_block"] = ("alu", sum(2 * min(s.n, 512) ** 2 * s.n // 3 for s in wl.inputs.values()), "TFLOP/s")
     tc_prep = [s for s in wl.inputs.values() if s.n > 512 and s.n % 4 == 0]
     per_step["chol_update"] = ("alu", sum(64 * s.n ** 2 for s in wl.inputs.values()) +
                                sum(s.n ** 3 // 3 for s in wl.inputs.values() if s not in tc_prep), "TFLOP/s")
-    per_step["chol_update_tc"] = ("tf32x3", sum(s.n ** 3 // 3 - 64 * s.n ** 2 for s in tc_prep), "TFLOP/s")
+    per_step["chol_update_tc"] = ("bf16x6", sum(s.n ** 3 // 3 for s in tc_prep), "TFLOP/s")
+    per_step["trtri_update_tc"] = ("bf16x6", sum(s.n ** 3 // 3 for s in tc_prep), "TFLOP/s")
     per_step["trtri_trmm_tc"] = ("tf32x3", sum(s.n ** 3 // 3 for s in tc_prep), "TFLOP/s")
     per_step["trtri_trmm"] = ("alu", sum(s.n ** 3 // 3 for s in wl.inputs.values() if s not in tc_prep), "TFLOP/s")
     return per_step
@@ -474,6 +476,12 @@ def roofline_entry(wl, name, launches, ms, steps, peaks, per_step):
         achieved = total / secs / 1e12
         peak = peaks["bf16_tflops_sustained"] / 3.0
         peak_note = f"fp32 via 3 fp16 passes: sustained bf16 / 3, {peaks['source']}"
+    elif bound == "bf16x6":
+        # fp32-accurate contraction as six bf16 products of three planes per operand
+        bound = "tensor"
+        achieved = total / secs / 1e12
+        peak = peaks["bf16_tflops_sustained"] / 6.0
+        peak_note = f"fp32 via 6 bf16 passes: sustained bf16 / 6, {peaks['source']}"
     elif bound == "alu":
         achieved = total / secs / 1e12
         peak = fp32_alu_tflops
@@ -705,14 +713,16 @@ def window_measure(args, peaks, steps, warmup):
     fwd = 2 * T * (2 * d * H * dh + 2 * d * Hkv * dh + 3 * d * f) + 2 * T * L * H * dh
     flop = 8 * fwd
     tf = flop / (ms / 1e3) / 1e12
-    if args.block_products:
-        # the projections as tf32x3 tensor-core products (the attention stays
-        # on the CUDA cores)
-        peak = peaks["bf16_tflops_sustained"] * (1.1 / 2.25) / 3.0
-        src, bound = f"fp32 via 3 tf32 passes: sustained bf16 x 1.1/2.25 / 3, {peaks['source']}", "tensor"
-    else:
-        peak = 152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
-        src, bound = "fp32 ALU: 152 SMs x 128 lanes x 2 x max clock", "alu"
+    # the projections on the tensor cores (bf16x6, or tf32x3 with
+    # --block-products 1), the attention on the CUDA cores: the peak is all the
+    # work over the two parts' least times
+    alu = 152 * 128 * 2 * peaks.get("sm_max_mhz", 2070.0) * 1e6 / 1e12
+    tensor = peaks["bf16_tflops_sustained"] * (1.1 / 2.25 / 3.0 if args.block_products else 1.0 / 6.0)
+    attn = 2 * T * L * H * dh
+    peak = fwd / ((fwd - attn) / tensor + attn / alu)
+    src = (f"projections at sustained bf16 {'x 1.1/2.25 / 3' if args.block_products else '/ 6'} ({peaks['source']}), "
+           "attention at the fp32 ALU peak (152 SMs x 128 lanes x 2 x max clock)")
+    bound = "alu"
     return {"kernel": "block_module_window", "d": d, "heads": H, "kv_heads": Hkv, "head_dim": dh, "ffn": f,
             "seqs": S, "seq_len": L, "block_products": args.block_products, "steps": steps, "ms_per_call": ms,
             "achieved": tf, "unit": "TFLOP/s", "peak": peak, "frac": tf / peak, "peak_source": src, "bound": bound}
@@ -756,7 +766,7 @@ def main():
     ap.add_argument("--seqs", type=int, default=2)
     ap.add_argument("--seq-len", type=int, default=2048)
     ap.add_argument("--block-products", type=int, choices=[0, 1], default=0,
-                    help="window: the block ops' products on tf32x3 tensor cores (1) or fp32 CUDA cores (0)")
+                    help="window: the block ops' products as bf16x6 (0, fp32 accuracy) or tf32x3 (1)")
     ap.add_argument("--n", type=int, default=2048)
     ap.add_argument("--m", type=int, default=1024)
     ap.add_argument("--tokens", type=int, default=65536)
