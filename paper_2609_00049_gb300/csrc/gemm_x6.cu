@@ -271,7 +271,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 
 // The three bf16 parts of v, rounded to nearest (a finite value whose first
 // part would round to infinity is truncated instead; the parts of a
-// non-finite value are the value and zeros).
+// non-finite value are the value and zeros, so that a product with an infinite
+// operand is infinite or, where the other's later parts are zero, NaN).
 __device__ __forceinline__ void split3(float v, __nv_bfloat16 &a, __nv_bfloat16 &b, __nv_bfloat16 &c) {
     a = __float2bfloat16_rn(v);
     float h = __bfloat162float(a);

@@ -30,3 +30,18 @@ def test_exact_on_integers_at_tile_edges(n, T, splits):
     assert torch.equal(H.double().cpu(), H0.double().cpu() + a.T @ a)
     assert torch.equal(D.double().cpu(), D0.double().cpu() + a.T @ a - b.T @ a)
     assert torch.equal(P, H)
+
+
+@pytest.mark.parametrize("off", [(1, 0), (0, 2), (3, 1)])
+def test_moments_at_any_word(off):
+    """H and D as views that begin at any 4-byte word of their buffers."""
+    n, T = 264, 5000
+    g = torch.Generator().manual_seed(off[0] * 4 + off[1])
+    Xh = torch.randint(-3, 4, (T, n), generator=g).to(torch.bfloat16).cuda()
+    Xf = torch.randint(-3, 4, (T, n), generator=g).to(torch.bfloat16).cuda()
+    H, D = (torch.zeros(n * n + 4, device="cuda")[o:o + n * n].view(n, n) for o in off)
+    ws = rq.workspace(rq.realq_hessian_workspace_size(n, T, rq.REALQ_BF16, True))
+    rq.realq_hessian_accumulate(Xh, H, D, Xf, ws=ws)
+    a, b = Xh.double().cpu(), Xf.double().cpu()
+    assert torch.equal(H.double().cpu(), a.T @ a)
+    assert torch.equal(D.double().cpu(), a.T @ a - b.T @ a)
