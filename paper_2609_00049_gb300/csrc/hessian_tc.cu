@@ -393,15 +393,17 @@ __device__ __forceinline__ void two_sum(float &s, float &e, float a) {
 // flight; the mirror image goes through shared memory, so that every access is
 // part of a row of float4 (n a multiple of 8; the caller's H and D, of which
 // only 4-byte alignment is asked, go word by word where either has no 16-byte
-// base: `vec` is 0).  Sums carry their rounding error: D is the small difference
+// base: VEC false).  Sums carry their rounding error: D is the small difference
 // of two large sums.  MS bounds the splits (4, 8 or 16), so that few splits take
 // few registers.
 constexpr int MAX_SPLITS = 16;
-__device__ __forceinline__ float4 row4(const float *p, int vec) {
-    return vec ? *reinterpret_cast<const float4 *>(p) : make_float4(p[0], p[1], p[2], p[3]);
+template <bool VEC>
+__device__ __forceinline__ float4 row4(const float *p) {
+    return VEC ? *reinterpret_cast<const float4 *>(p) : make_float4(p[0], p[1], p[2], p[3]);
 }
-__device__ __forceinline__ void put4(float *p, float4 v, int vec) {
-    if (vec) {
+template <bool VEC>
+__device__ __forceinline__ void put4(float *p, float4 v) {
+    if (VEC) {
         *reinterpret_cast<float4 *>(p) = v;
     } else {
         p[0] = v.x;
@@ -410,9 +412,9 @@ __device__ __forceinline__ void put4(float *p, float4 v, int vec) {
         p[3] = v.w;
     }
 }
-template <bool CROSS, int MS, int TILE>
+template <bool CROSS, int MS, int TILE, bool VEC>
 __global__ void __launch_bounds__(256) hess_tc_reduce_kernel(int64_t n, int splits, const float *part,
-                                                             const float *partC, float *H, float *D, int vec) {
+                                                             const float *partC, float *H, float *D) {
     constexpr int TPR = TILE / 4, ROWS = 256 / TPR, PER = TILE / ROWS;   // threads per row, rows per pass, passes
     __shared__ float th[TILE][TILE + 1], tl[TILE][TILE + 1];
     int bi = (int)((sqrt(8.0 * (double)blockIdx.x + 1.0) - 1.0) * 0.5);
@@ -437,16 +439,16 @@ __global__ void __launch_bounds__(256) hess_tc_reduce_kernel(int64_t n, int spli
         if (CROSS) {
             float x[4] = {}, xe[4] = {};
             sum(partC + at, x, xe);
-            float4 d = row4(D + at, vec);
+            float4 d = row4<VEC>(D + at);
             d.x += (s[0] - x[0]) + (e[0] - xe[0]);
             d.y += (s[1] - x[1]) + (e[1] - xe[1]);
             d.z += (s[2] - x[2]) + (e[2] - xe[2]);
             d.w += (s[3] - x[3]) + (e[3] - xe[3]);
-            put4(D + at, d, vec);
+            put4<VEC>(D + at, d);
         }
-        float4 h = row4(H + at, vec);
+        float4 h = row4<VEC>(H + at);
         h.x += s[0] + e[0]; h.y += s[1] + e[1]; h.z += s[2] + e[2]; h.w += s[3] + e[3];
-        put4(H + at, h, vec);
+        put4<VEC>(H + at, h);
     };
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
@@ -639,17 +641,18 @@ static realq_status_t hess_tc_launch(cudaStream_t s, int64_t n, int64_t T, const
         return REALQ_OK;
     }
     REALQ_TRY(launch(hess_grid(n, true, XC != nullptr), nullptr, nullptr, 1.f, name));
+    const bool vec = ((reinterpret_cast<uintptr_t>(H) | (XC ? reinterpret_cast<uintptr_t>(D) : 0)) & 15) == 0;
     // 64 x 64 tiles where they fill the SMs twice over, else 32 x 32 (n = 1024:
     // 136 tiles took 24 us, 528 take 11)
-    const int tile = n >= 1536 ? 64 : 32;
+    const int tile = vec && n >= 1536 ? 64 : 32;
     const int64_t nb = ceil_div(n, tile);
     const unsigned tiles = (unsigned)(nb * (nb + 1) / 2);
-    const int vec = ((reinterpret_cast<uintptr_t>(H) | (XC ? reinterpret_cast<uintptr_t>(D) : 0)) & 15) == 0;
     auto reduce = [&](auto cross, auto ms) {
         constexpr bool CR = decltype(cross)::value;
         constexpr int MS = decltype(ms)::value;
-        if (tile == 64) hess_tc_reduce_kernel<CR, MS, 64><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D, vec);
-        else hess_tc_reduce_kernel<CR, MS, 32><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D, vec);
+        if (!vec) hess_tc_reduce_kernel<CR, MS, 32, false><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D);
+        else if (tile == 64) hess_tc_reduce_kernel<CR, MS, 64, true><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D);
+        else hess_tc_reduce_kernel<CR, MS, 32, true><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D);
     };
     auto by_splits = [&](auto cross) {
         if (splits <= 4) reduce(cross, std::integral_constant<int, 4>());
