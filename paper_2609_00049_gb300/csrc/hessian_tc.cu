@@ -604,8 +604,7 @@ static realq_status_t hess_tc_launch(cudaStream_t s, int64_t n, int64_t T, const
     map(&mapC, XC ? XC : XA);
     if (cr != CUDA_SUCCESS) return fail(REALQ_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)cr);
     const size_t per = (size_t)n * n * sizeof(float) * (XC ? 2 : 1);
-    // (the symmetric product's count also with cross tiles: H then has the same
-    // bits whether or not D is asked for)
+    // (the symmetric product's count also with cross tiles)
     int splits = tc_splits(hess_grid(n, true, false), T, sms);
     if (splits > 1 && (ws == nullptr || ws_bytes < 2 * per)) splits = 1;
     if (splits > 1 && (size_t)splits * per > ws_bytes) splits = (int)(ws_bytes / per);   // (at most the plan's)
@@ -669,7 +668,12 @@ static realq_status_t hess_tc_launch(cudaStream_t s, int64_t n, int64_t T, const
 
 realq_status_t hessian_syrk_tc(cudaStream_t s, int64_t n, int64_t T, const void *X, const void *Xfp, float *H, float *D,
                                int *err, void *ws, size_t ws_bytes, int sms) {
-    return hess_tc_launch(s, n, T, X, nullptr, Xfp, H, D, err, ws, ws_bytes, sms, "hessian_syrk_tc", CHUNK_STAGES);
+    // D is the small difference of two large sums, which magnifies the
+    // accumulator's rounding: with it 512 tokens per pass (n = 2056, T = 50,001:
+    // 690 us and 5e-6 to 7e-6 of D's scale against 64 bits; 1024: 636 us and
+    // 9e-6 to 11e-6)
+    return hess_tc_launch(s, n, T, X, nullptr, Xfp, H, D, err, ws, ws_bytes, sms, "hessian_syrk_tc",
+                          Xfp ? CHUNK_STAGES / 2 : CHUNK_STAGES);
 }
 
 realq_status_t hessian_pair_tc(cudaStream_t s, int64_t n, int64_t T, const void *XA, const void *XB, float *H, int *err,
