@@ -20,9 +20,9 @@
 // last place per accumulated MMA, in one direction, so a TMEM accumulator that
 // takes all 2^18 tokens of a calibration set (2^14 MMAs) drifts by ~1e-3 of
 // the entry.  The accumulation is therefore promoted: TMEM holds two 128 x 256
-// accumulators (per CTA), the MMA issuer switches between them every 1024 tokens (512 halve the error but cost 6 %), and
-// the eight drain warps add each finished chunk into fp32 registers (IEEE
-// adds) while the other accumulator fills.
+// accumulators (per CTA), the MMA issuer switches between them every 512 tokens
+// (CHUNK_STAGES), and the eight drain warps add each finished chunk into fp32
+// registers (IEEE adds) while the other accumulator fills.
 //
 // Roles (320 threads per CTA): warp 8 lane 0 issues the CTA's TMA loads into a
 // STAGES-deep ring (counted on the leader's barriers), warp 9 lane 0 of the
@@ -63,7 +63,13 @@ constexpr int TM = 128;                          // tile rows of one CTA (channe
 constexpr int TN = 256;                          // tile rows of the pair, and tile columns (channels j)
 constexpr int KSTAGE = 64;                       // tokens per pipeline stage
 constexpr int STAGES = 6;
-constexpr int CHUNK_STAGES = 16;                 // default: 1024 tokens per TMEM accumulator pass
+// 512 tokens per TMEM accumulator pass, with and without D: H then has the same
+// bits whether or not D is asked for.  D, the small difference of two large
+// sums, magnifies the accumulator's rounding and sets the length (n = 2056, T =
+// 50,001: 690 us and 5e-6 to 7e-6 of D's scale against 64 bits; with 1024 tokens
+// 636 us and 9e-6 to 11e-6).  H alone takes 6 % longer for it, at half the error:
+// n = 8192, T = 65,536: 3.07 -> 3.26 ms, 2.2e-6 -> 1.1e-6.
+constexpr int CHUNK_STAGES = 8;
 constexpr int DRAIN_WARPS = 8;                   // two per TMEM lane quarter, 128 columns each
 constexpr int THREADS = (DRAIN_WARPS + 2) * 32;  // + the TMA warp and the MMA warp
 constexpr int BOX_BYTES = 64 * KSTAGE * 2;       // one TMA box (64 channels x 64 tokens)
@@ -562,7 +568,7 @@ bool hessian_tc_eligible(int64_t n, int64_t T, const void *X) {
 // share of a tile's time + a CTA's fixed cost) + the partial sums' traffic,
 // in microseconds (a 64-token stage of a pair is 0.29 us at 1.75 GHz; a CTA's
 // start, fill and epilogue about 8 us; a partial 256 x 256 tile written and
-// read at 5 TB/s).  At least 1024 tokens per split (one promoted chunk) and at
+// read at 5 TB/s).  At least 1024 tokens per split (two accumulator passes) and at
 // most 16 splits.
 static int tc_splits(const HessGrid &g, int64_t T, int sms) {
     const int64_t full = (g.nsym ? (int64_t)g.nf * (g.nf + 1) / 2 : 0) + (g.ncross ? (int64_t)g.nf * g.nf : 0);
@@ -668,12 +674,7 @@ static realq_status_t hess_tc_launch(cudaStream_t s, int64_t n, int64_t T, const
 
 realq_status_t hessian_syrk_tc(cudaStream_t s, int64_t n, int64_t T, const void *X, const void *Xfp, float *H, float *D,
                                int *err, void *ws, size_t ws_bytes, int sms) {
-    // D is the small difference of two large sums, which magnifies the
-    // accumulator's rounding: with it 512 tokens per pass (n = 2056, T = 50,001:
-    // 690 us and 5e-6 to 7e-6 of D's scale against 64 bits; 1024: 636 us and
-    // 9e-6 to 11e-6)
-    return hess_tc_launch(s, n, T, X, nullptr, Xfp, H, D, err, ws, ws_bytes, sms, "hessian_syrk_tc",
-                          Xfp ? CHUNK_STAGES / 2 : CHUNK_STAGES);
+    return hess_tc_launch(s, n, T, X, nullptr, Xfp, H, D, err, ws, ws_bytes, sms, "hessian_syrk_tc", CHUNK_STAGES);
 }
 
 realq_status_t hessian_pair_tc(cudaStream_t s, int64_t n, int64_t T, const void *XA, const void *XB, float *H, int *err,

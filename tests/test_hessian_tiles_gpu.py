@@ -45,3 +45,18 @@ def test_moments_at_any_word(off):
     a, b = Xh.double().cpu(), Xf.double().cpu()
     assert torch.equal(H.double().cpu(), a.T @ a)
     assert torch.equal(D.double().cpu(), a.T @ a - b.T @ a)
+
+
+@pytest.mark.parametrize("splits", [True, False])
+@pytest.mark.parametrize("n,T", [(128, 65536), (264, 9000), (512, 20000), (2056, 3000)])
+def test_h_has_the_same_bits_with_and_without_d(n, T, splits):
+    """Real-valued activations over several accumulator passes, where another
+    order of the sums gives other bits (above, every order is exact)."""
+    g = torch.Generator().manual_seed(n + T)
+    Xh = torch.randn(T, n, generator=g).to(torch.bfloat16).cuda()
+    Xf = torch.randn(T, n, generator=g).to(torch.bfloat16).cuda()
+    ws = rq.workspace(rq.realq_hessian_workspace_size(n, T, rq.REALQ_BF16, True)) if splits else None
+    H, D, P = (torch.zeros(n, n, device="cuda") for _ in range(3))
+    rq.realq_hessian_accumulate(Xh, H, D, Xf, ws=ws)
+    rq.realq_hessian_accumulate(Xh, P, ws=ws)
+    assert torch.equal(P, H)
