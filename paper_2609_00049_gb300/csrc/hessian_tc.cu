@@ -43,8 +43,9 @@
 // moment of the perturbed-input surrogate is D = X̂ᵀX̂ - XᵀX̂.  With token splits
 // both products run in one launch over the same splits and the reduction
 // subtracts their sums (kept in two floats each) before it adds to D, so that
-// little of D is lost to the size of its two parts; without splits the
-// symmetric pass also adds into D and a second launch subtracts.
+// little of D is lost to the size of its two parts; without splits, or where the
+// workspace holds one product's partial sums only, the symmetric sum is also
+// added to D and a second launch subtracts.
 // Every wait is bounded; on a timeout the tile is written as NaN (so the
 // factorisation of H reports a non-finite pivot), the workspace status word
 // gets ST_TIMEOUT, and the kernel still frees TMEM and returns.
@@ -609,8 +610,10 @@ static realq_status_t hess_tc_launch(cudaStream_t s, int64_t n, int64_t T, const
     map(&mapB, XB ? XB : XA);
     map(&mapC, XC ? XC : XA);
     if (cr != CUDA_SUCCESS) return fail(REALQ_ERR_CUDA, "cuTensorMapEncodeTiled failed (%d)", (int)cr);
-    const size_t per = (size_t)n * n * sizeof(float) * (XC ? 2 : 1);
-    // (the symmetric product's count also with cross tiles)
+    // the symmetric product's count also with cross tiles, by the room for its
+    // own partial sums: H then has the same bits whether or not D is asked for,
+    // whatever the workspace
+    const size_t per = (size_t)n * n * sizeof(float);
     int splits = tc_splits(hess_grid(n, true, false), T, sms);
     if (splits > 1 && (ws == nullptr || ws_bytes < 2 * per)) splits = 1;
     if (splits > 1 && (size_t)splits * per > ws_bytes) splits = (int)(ws_bytes / per);   // (at most the plan's)
@@ -619,7 +622,10 @@ static realq_status_t hess_tc_launch(cudaStream_t s, int64_t n, int64_t T, const
     splits = (int)((T + tper - 1) / tper);
     REALQ_TRY(set_smem_limit(reinterpret_cast<const void *>(hess_tc_kernel), SMEM_BYTES));
     float *part = splits > 1 ? static_cast<float *>(ws) : nullptr;
-    float *partC = part ? part + (size_t)splits * n * n : nullptr;
+    // both products' partial sums side by side where the workspace holds them,
+    // else one after the other
+    const bool both = XC && 2 * (size_t)splits * per <= ws_bytes;
+    float *partC = both ? part + (size_t)splits * n * n : part;
     auto launch = [&](const HessGrid &g, float *o, float *o2, float sign, const char *who) -> realq_status_t {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)(2 * (g.nsym + g.ncross)), (unsigned)splits);
@@ -645,31 +651,35 @@ static realq_status_t hess_tc_launch(cudaStream_t s, int64_t n, int64_t T, const
         if (XC) REALQ_TRY(launch(hess_grid(n, false, true), D, nullptr, -1.f, "hessian_cross_tc"));
         return REALQ_OK;
     }
-    REALQ_TRY(launch(hess_grid(n, true, XC != nullptr), nullptr, nullptr, 1.f, name));
+    REALQ_TRY(launch(hess_grid(n, true, both), nullptr, nullptr, 1.f, name));
     const bool vec = ((reinterpret_cast<uintptr_t>(H) | (XC ? reinterpret_cast<uintptr_t>(D) : 0)) & 15) == 0;
     // 64 x 64 tiles where they fill the SMs twice over, else 32 x 32 (n = 1024:
     // 136 tiles took 24 us, 528 take 11)
     const int tile = vec && n >= 1536 ? 64 : 32;
     const int64_t nb = ceil_div(n, tile);
     const unsigned tiles = (unsigned)(nb * (nb + 1) / 2);
-    auto reduce = [&](auto cross, auto ms) {
+    auto reduce = [&](auto cross, auto ms, float *h) {
         constexpr bool CR = decltype(cross)::value;
         constexpr int MS = decltype(ms)::value;
-        if (!vec) hess_tc_reduce_kernel<CR, MS, 32, false><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D);
-        else if (tile == 64) hess_tc_reduce_kernel<CR, MS, 64, true><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D);
-        else hess_tc_reduce_kernel<CR, MS, 32, true><<<tiles, 256, 0, s>>>(n, splits, part, partC, H, D);
+        if (!vec) hess_tc_reduce_kernel<CR, MS, 32, false><<<tiles, 256, 0, s>>>(n, splits, part, partC, h, D);
+        else if (tile == 64) hess_tc_reduce_kernel<CR, MS, 64, true><<<tiles, 256, 0, s>>>(n, splits, part, partC, h, D);
+        else hess_tc_reduce_kernel<CR, MS, 32, true><<<tiles, 256, 0, s>>>(n, splits, part, partC, h, D);
     };
-    auto by_splits = [&](auto cross) {
-        if (splits <= 4) reduce(cross, std::integral_constant<int, 4>());
-        else if (splits <= 8) reduce(cross, std::integral_constant<int, 8>());
-        else reduce(cross, std::integral_constant<int, MAX_SPLITS>());
+    auto by_splits = [&](auto cross, float *h) -> realq_status_t {
+        {
+            Launch L("hessian_reduce", s);
+            if (splits <= 4) reduce(cross, std::integral_constant<int, 4>(), h);
+            else if (splits <= 8) reduce(cross, std::integral_constant<int, 8>(), h);
+            else reduce(cross, std::integral_constant<int, MAX_SPLITS>(), h);
+        }
+        return check_launch("hessian_reduce");
     };
-    {
-        Launch L("hessian_reduce", s);
-        if (XC) by_splits(std::true_type());
-        else by_splits(std::false_type());
-    }
-    return check_launch("hessian_reduce");
+    if (both) return by_splits(std::true_type(), H);
+    REALQ_TRY(by_splits(std::false_type(), H));
+    if (!XC) return REALQ_OK;
+    REALQ_TRY(by_splits(std::false_type(), D));
+    REALQ_TRY(launch(hess_grid(n, false, true), nullptr, nullptr, -1.f, "hessian_cross_tc"));
+    return hessian_reduce(s, n, splits, partC, D, 1);
 }
 
 realq_status_t hessian_syrk_tc(cudaStream_t s, int64_t n, int64_t T, const void *X, const void *Xfp, float *H, float *D,

@@ -60,3 +60,20 @@ def test_h_has_the_same_bits_with_and_without_d(n, T, splits):
     rq.realq_hessian_accumulate(Xh, H, D, Xf, ws=ws)
     rq.realq_hessian_accumulate(Xh, P, ws=ws)
     assert torch.equal(P, H)
+
+
+@pytest.mark.parametrize("n,T", [(264, 9000), (512, 20000)])
+def test_h_has_the_same_bits_in_a_workspace_sized_without_d(n, T):
+    """Room for one product's partial sums only: H as without D, and D within
+    the bound of its two parts' fp32 sums (each about sqrt(T) units of 2^-24 of
+    the diagonal's scale T; 1e-5 T leaves a factor of ten)."""
+    g = torch.Generator().manual_seed(n + T)
+    Xh = torch.randn(T, n, generator=g).to(torch.bfloat16).cuda()
+    Xf = torch.randn(T, n, generator=g).to(torch.bfloat16).cuda()
+    ws = rq.workspace(rq.realq_hessian_workspace_size(n, T, rq.REALQ_BF16, False))
+    H, D, P = (torch.zeros(n, n, device="cuda") for _ in range(3))
+    rq.realq_hessian_accumulate(Xh, H, D, Xf, ws=ws)
+    rq.realq_hessian_accumulate(Xh, P, ws=ws)
+    assert torch.equal(P, H)
+    a, b = Xh.double().cpu(), Xf.double().cpu()
+    assert (D.double().cpu() - (a.T @ a - b.T @ a)).abs().max().item() <= 1e-5 * T
