@@ -46,9 +46,10 @@
 // little of D is lost to the size of its two parts; without splits, or where the
 // workspace holds one product's partial sums only, the symmetric sum is also
 // added to D and a second launch subtracts.
-// Every wait is bounded; on a timeout the tile is written as NaN (so the
-// factorisation of H reports a non-finite pivot), the workspace status word
-// gets ST_TIMEOUT, and the kernel still frees TMEM and returns.
+// Every wait is bounded; on a timeout in either CTA of a pair the whole tile is
+// written as NaN (so the factorisation of H reports a non-finite pivot), the
+// workspace status word gets ST_TIMEOUT, and the kernel still frees TMEM and
+// returns.
 #include "kernels.cuh"
 #include "tc.cuh"
 
@@ -226,8 +227,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             // mapB, the other way round when the tile is stored transposed
             const CUtensorMap *ma = !tl.cross ? &mapA : (tl.swap ? &mapB : &mapC);
             const CUtensorMap *mb = tl.cross && tl.swap ? &mapC : &mapB;
-            int it = 0;
-            for (; it < nk; ++it) {
+            for (int it = 0; it < nk; ++it) {
                 const int s = it % STAGES;
                 const uint32_t r = (uint32_t)(it / STAGES);
                 if (!tc::mbar_wait(tc::smem_u32(&empty[s]), (r & 1u) ^ 1u, abort_flag)) {
@@ -242,14 +242,6 @@ __global__ void __launch_bounds__(THREADS, 1)
                 tc::tma_load_2d_pair(a, ma, fb, i0, y);
                 tc::tma_load_2d_pair(a + BOX_BYTES, ma, fb, i0 + 64, y);
                 for (int q = 0; q < bboxes; ++q) tc::tma_load_2d_pair(a + A_BYTES + q * BOX_BYTES, mb, fb, jl + 64 * q, y);
-            }
-            // on abort, let the copies already issued land before the CTAs
-            // exit (the leader waits for both, before the cluster barrier)
-            if (*abort_flag && leader) {
-                int never = 0;
-                for (int k = (it > STAGES ? it - STAGES : 0); k < it; ++k)
-                    tc::mbar_wait(tc::smem_u32(&full[k % STAGES]), (uint32_t)(k / STAGES) & 1u, &never,
-                                  100000000ull);
             }
         }
     } else if (warp == DRAIN_WARPS + 1) {
@@ -284,7 +276,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                     }
                     tc::mma_commit_pair(tc::smem_u32(&empty[s]));
                 }
-                tc::mma_commit_pair(tc::smem_u32(&accf[b]));
+                // (a chunk cut short is not announced)
+                if (!*abort_flag) tc::mma_commit_pair(tc::smem_u32(&accf[b]));
             }
             // every MMA issued has retired before TMEM is freed
             tc::mma_commit_pair(tc::smem_u32(drain));
@@ -318,7 +311,19 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
     }
     __syncwarp();
-    const bool all_good = __syncthreads_and(good && !*abort_flag) != 0;
+    // both CTAs of the pair take the same outcome: either one's failure
+    const bool mine = __syncthreads_and(good && !*abort_flag) != 0;
+    if (!mine && threadIdx.x == 0) tc::st_cluster_u32(tc::mapa(tc::smem_u32((const void *)abort_flag), rank ^ 1u), 1u);
+    __syncwarp();
+    tc::cluster_sync();
+    const bool all_good = mine && !*abort_flag;
+    if (!all_good) {
+        // the copies already issued land before the ring is used or the CTA
+        // exits; they count on the leader's barriers, of which an abort may
+        // leave some unarmed, so both CTAs wait by the clock
+        if (threadIdx.x == 0) tc::wait_ns(100000000ull);
+        __syncthreads();
+    }
 
     // ---------------- epilogue (drain warps) ----------------
     // Each drain warp owns a 32-row x 128-column piece, in 128-row block ib and
@@ -372,7 +377,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                             for (int q = 0; q < 16; ++q) old[q] = direct && gi0 + h + q < n ? d[(h + q) * n] : 0.f;
 #pragma unroll
                             for (int q = 0; q < 16; ++q)
-                                if (gi0 + h + q < n) d[(h + q) * n] = old[q] + st[(h + q) * 33 + lane];
+                                if (gi0 + h + q < n)
+                                    d[(h + q) * n] = all_good ? old[q] + st[(h + q) * 33 + lane] : v[0];
                         }
                     }
                     __syncwarp();
