@@ -211,9 +211,13 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// arrive on a barrier of another CTA of the cluster (address from mapa)
+// Arrive on a barrier of another CTA of the cluster (address from mapa).  For
+// "TMEM has been read" (tcgen05.wait::ld and the fence before it): nothing in
+// memory is handed over, so the default CTA scope does.  .release.cluster held
+// the MMA issuer up by about 1 us per accumulator (two groups' weighted Hessians,
+// 128 tokens per accumulator, n = 1024, T = 131,072: 1481 us, 1055 without).
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // a word of another CTA's shared memory (address from mapa)
 __device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
