@@ -331,12 +331,15 @@ __global__ void __launch_bounds__(THREADS, 1)
     // and mirrored, jb == ib (the diagonal block) is added in full, jb > ib lies
     // above the diagonal and is left to the CTA that holds its mirror image (a
     // swapped tile lies above it as a whole and is added mirrored).
+    // (The sums leave their registers here at once: with both directions written
+    // from registers the kernel spilled 388 bytes a thread, in the drain loop too:
+    // n = 2056, T = 50,001 with D 661 us, 568 without.)
     if (warp < DRAIN_WARPS && (nk > 0 || !all_good)) {
         const bool direct = part == nullptr;
         const int ib = 2 * tl.ti + (int)rank, jb = 2 * tl.tj + (warp >> 2);
         const bool plain = tl.cross ? !tl.swap : (tl.swap ? direct : jb <= ib);              // at [i][j]
         const bool turned = tl.cross ? tl.swap : (tl.swap || (direct && jb < ib));           // at [j][i]
-        const float mul = tl.cross ? sign : 1.f;
+        const float mul = tl.cross ? sign : 1.f, nan = __int_as_float(0x7fc00000);
         float *o1 = direct ? H : (tl.cross ? partC : part) + (int64_t)blockIdx.y * n * n;
         float *o2 = direct && !tl.cross ? H2 : nullptr;
         float *st = reinterpret_cast<float *>(smem) + warp * 32 * 33;
@@ -345,45 +348,29 @@ __global__ void __launch_bounds__(THREADS, 1)
         for (int c0 = 0; c0 < 128; c0 += 32) {
             const int64_t gj0 = (int64_t)tl.tj * TN + (warp >> 2) * 128 + c0;
             if (gj0 >= n || gi0 >= n) continue;
-            float v[32];
 #pragma unroll
-            for (int q = 0; q < 32; ++q) v[q] = all_good ? mul * acc[c0 + q] : __int_as_float(0x7fc00000);
+            for (int q = 0; q < 32; ++q) st[lane * 33 + q] = mul * acc[c0 + q];
+            __syncwarp();
 #pragma unroll 1
             for (int w = 0; w < 2; ++w) {
                 float *o = w ? o2 : o1;
                 if (!o) break;
-                if (turned && gi < n) {
-                    float *d = o + gj0 * n + gi;
-#pragma unroll
-                    for (int h = 0; h < 32; h += 16) {
+                // 32 x 16 of the piece at a time: its old values first
+                auto add = [&](float *d, int64_t at, const float *src, int step) {
+#pragma unroll 1
+                    for (int h = 0; h < 32; h += 16, d += 16 * n, at += 16, src += 16 * step) {
                         float old[16];
 #pragma unroll
-                        for (int q = 0; q < 16; ++q) old[q] = direct && gj0 + h + q < n ? d[(h + q) * n] : 0.f;
+                        for (int q = 0; q < 16; ++q) old[q] = direct && at + q < n ? d[q * n] : 0.f;
 #pragma unroll
                         for (int q = 0; q < 16; ++q)
-                            if (gj0 + h + q < n) d[(h + q) * n] = old[q] + v[h + q];
+                            if (at + q < n) d[q * n] = all_good ? old[q] + src[q * step] : nan;
                     }
-                }
-                if (plain) {
-#pragma unroll
-                    for (int q = 0; q < 32; ++q) st[lane * 33 + q] = v[q];
-                    __syncwarp();
-                    if (gj0 + lane < n) {
-                        float *d = o + gi0 * n + gj0 + lane;
-#pragma unroll 1
-                        for (int h = 0; h < 32; h += 16) {
-                            float old[16];
-#pragma unroll
-                            for (int q = 0; q < 16; ++q) old[q] = direct && gi0 + h + q < n ? d[(h + q) * n] : 0.f;
-#pragma unroll
-                            for (int q = 0; q < 16; ++q)
-                                if (gi0 + h + q < n)
-                                    d[(h + q) * n] = all_good ? old[q] + st[(h + q) * 33 + lane] : v[0];
-                        }
-                    }
-                    __syncwarp();
-                }
+                };
+                if (turned && gi < n) add(o + gj0 * n + gi, gj0, st + lane * 33, 1);
+                if (plain && gj0 + lane < n) add(o + gi0 * n + gj0 + lane, gi0, st + lane, 33);
             }
+            __syncwarp();
         }
     }
     if (!all_good && threadIdx.x == 0 && err) atomicOr(err, ST_TIMEOUT);
