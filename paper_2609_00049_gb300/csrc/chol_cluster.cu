@@ -32,7 +32,9 @@
 // and dependent FMAs.
 #include "kernels.cuh"
 
+#include <map>
 #include <mutex>
+#include <utility>
 
 namespace realq {
 namespace {
@@ -583,18 +585,19 @@ __global__ void __launch_bounds__(TH, 1) chol_cluster_kernel(int64_t ld, float *
     write_held(cta, nc);
 }
 
-// CTAs of the cluster: 16 where the device places such a cluster, else 8
-// (held slices: at most 14 of a row block over 7 CTAs, so 2 each)
-int cluster_ctas(bool vec) {
+// CTAs of the cluster: 16 where the current device places such a cluster, else
+// 8 (held slices: at most 14 of a row block over 7 CTAs, so 2 each).  The
+// permission for more than 8 CTAs and the answer both belong to a device: they
+// are set and asked once per device and kernel.
+realq_status_t cluster_ctas(const void *fn, int *ctas) {
+    int dev = 0;
+    REALQ_CUDA_TRY(cudaGetDevice(&dev));
     static std::mutex mu;
-    static int best[2] = {0, 0};
+    static std::map<std::pair<int, const void *>, int> best;
     std::lock_guard<std::mutex> lk(mu);
-    int &b = best[vec ? 1 : 0];
-    if (b) return b;
-    const void *fn = vec ? reinterpret_cast<const void *>(chol_cluster_kernel<true>)
-                         : reinterpret_cast<const void *>(chol_cluster_kernel<false>);
-    b = 8;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+    int &b = best[{dev, fn}];
+    if (!b) {
+        b = 8;
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(16);
         cfg.blockDim = dim3(TH);
@@ -606,10 +609,15 @@ int cluster_ctas(bool vec) {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n > 0) b = 16;
+        if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess) {
+            if (n > 0) b = 16;
+        } else {
+            cudaGetLastError();
+        }
     }
-    cudaGetLastError();
-    return b;
+    *ctas = b;
+    return REALQ_OK;
 }
 
 }  // namespace
@@ -622,7 +630,8 @@ realq_status_t chol_inv_block(cudaStream_t s, int64_t ld, float *A, int64_t n, i
                          : reinterpret_cast<const void *>(chol_cluster_kernel<false>);
     REALQ_TRY(set_smem_limit(fn, (int)sizeof(Sm)));
     // one piece has no panel, no update and no row of U beside it
-    const int nc = n <= NB ? 1 : cluster_ctas(vec);
+    int nc = 1;
+    if (n > NB) REALQ_TRY(cluster_ctas(fn, &nc));
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)nc);
     cfg.blockDim = dim3(TH);
