@@ -227,10 +227,14 @@ realq_status_t run(cudaStream_t s, int64_t n, int64_t T, const TX *X, const TX *
     float *partH = static_cast<float *>(ws);
     float *partD = partH + (size_t)splits * n * n;
     const int direct = splits == 1;
-    // 32 x 32 tiles while the 128 x 128 ones would leave SMs idle (both give
-    // the same bits)
+    // 32 x 32 tiles while the 128 x 128 ones would leave SMs idle (both give the
+    // same bits).  Without vector loads only while they leave a fifth of them
+    // idle: n = 2047, T = 4000 takes 718 us as 136 large tiles and 812 as small
+    // ones, n = 1919 (120 large ones) 717 and 713; with them n = 2048 takes 707
+    // and 685.
     const int nts = ceil_div(n, SB);
     const bool vec = n % 4 == 0 && ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(Xf)) & 15) == 0;
+    const auto small_pays = [&](int64_t tiles) { return vec ? tiles < num_sms() : 5 * tiles < 4 * num_sms(); };
     auto small = [&](auto mode, const TX *xf, float *o, float *p) {
         constexpr int M = decltype(mode)::value;
         const dim3 g((unsigned)(M == 0 ? (int64_t)nts * (nts + 1) / 2 : (int64_t)nts * nts), splits);
@@ -240,7 +244,7 @@ realq_status_t run(cudaStream_t s, int64_t n, int64_t T, const TX *X, const TX *
     if (H) {
         {
             Launch L("hessian_syrk_simt", s);
-            if (lower * splits < num_sms())
+            if (small_pays(lower * splits))
                 small(std::integral_constant<int, 0>(), nullptr, H, partH);
             else
                 hess_kernel<TX, 0><<<dim3((unsigned)lower, splits), THREADS, 0, s>>>(n, T, X, nullptr, H, partH, tper,
@@ -252,7 +256,7 @@ realq_status_t run(cudaStream_t s, int64_t n, int64_t T, const TX *X, const TX *
     if (Xf) {
         {
             Launch L("hessian_cross_simt", s);
-            if ((int64_t)nt * nt * splits < num_sms())
+            if (small_pays((int64_t)nt * nt * splits))
                 small(std::integral_constant<int, 1>(), Xf, D, partD);
             else
                 hess_kernel<TX, 1><<<dim3((unsigned)((int64_t)nt * nt), splits), THREADS, 0, s>>>(n, T, X, Xf, D, partD,
