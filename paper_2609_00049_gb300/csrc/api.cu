@@ -11,9 +11,8 @@
 #include <cstring>
 #include <map>
 #include <mutex>
-#include <set>
-#include <tuple>
 #include <string>
+#include <utility>
 #include <vector>
 
 namespace realq {
@@ -46,12 +45,13 @@ realq_status_t set_smem_limit(const void *kernel, int bytes) {
     int dev = 0;
     REALQ_CUDA_TRY(cudaGetDevice(&dev));
     static std::mutex mu;
-    static std::set<std::tuple<const void *, int, int>> done;
+    static std::map<std::pair<const void *, int>, int> limit;
     std::lock_guard<std::mutex> lk(mu);
-    const auto key = std::make_tuple(kernel, dev, bytes);
-    if (done.count(key)) return REALQ_OK;
+    // (never lowered: another width of the same kernel may have asked for more)
+    int &have = limit[{kernel, dev}];
+    if (have >= bytes) return REALQ_OK;
     REALQ_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    done.insert(key);
+    have = bytes;
     return REALQ_OK;
 }
 
