@@ -11,8 +11,9 @@
 // (chol_cluster.cu).  Wider inputs are blocked by 512: the cluster factors and
 // inverts each diagonal block, and everything beside it is a product of depth
 // 512 with fp32 accuracy on the tensor cores (gemm_x6.cu), spread over three
-// streams (prepare_blocked below).  The allocation-free entry point, whose
-// scratch has no room for operand planes, keeps 64-wide steps on the CUDA
+// streams (prepare_blocked below).  The allocation-free entry point takes the
+// same steps on one stream, with blocks as deep as its scratch has room for
+// operand planes; beyond that (n > 21824) it keeps 64-wide steps on the CUDA
 // cores (prepare_steps).  A pivot that is not positive (or not finite) records
 // its column in the workspace status word; prepare reads it once at the end,
 // the deferred variant leaves it for realq_prepare_status (a captured step
@@ -292,15 +293,31 @@ constexpr size_t prepare_bytes(int64_t n) {
     return align256(sizeof(int)) + align256(sizeof(float)) + align256((size_t)NB * NB * sizeof(float)) +
            align256((size_t)n * NB * sizeof(float));
 }
-// Operand planes of the blocked preparation (three bf16 planes each, 512
-// terms deep): U_KK, the panel A[0:k0, K] before its solve, kPanels panels
-// R[0:k0, K] (a step's updates may still read the earlier ones), the row block
-// of U before its product with U_KK, and its transpose after it.
+// Operand planes of the blocked preparation (three bf16 planes each, pb terms
+// deep; pb = PB with a workspace): U_KK, the panel A[0:k0, K] before its solve,
+// kPanels panels R[0:k0, K] (a step's updates may still read the earlier ones),
+// the row block of U before its product with U_KK, and its transpose after it.
 constexpr int64_t PB = kCholBlock;
 constexpr int kPanels = 3;
-constexpr size_t planes_bytes(int64_t rows) { return align256((size_t)rows * PB * 3 * sizeof(__nv_bfloat16)); }
+constexpr size_t planes_bytes(int64_t rows, int64_t pb) {
+    return align256((size_t)rows * pb * 3 * sizeof(__nv_bfloat16));
+}
 constexpr size_t blocked_bytes(int64_t n) {
-    return n <= PB ? 0 : planes_bytes(PB) + (size_t)(1 + kPanels + 2) * planes_bytes(n);
+    return n <= PB ? 0 : planes_bytes(PB, PB) + (size_t)(1 + kPanels + 2) * planes_bytes(n, PB);
+}
+// On one stream a step needs U_KK and n rows beside it: its panel (before the
+// solve, then after it) over the k0 rows above the block, and its row block (S,
+// then U) over the n - k0 columns from the block on.
+constexpr size_t compact_bytes(int64_t n, int64_t pb) { return planes_bytes(pb, pb) + planes_bytes(n, pb); }
+// The deepest blocks whose planes fit `bytes` on one stream (0: none).  The
+// allocation-free entry point's 8.4 MB hold 512 columns up to n = 2224, 256 up to
+// 5216, 128 up to 10816 and 64 up to 21824; against 64-wide steps on the CUDA
+// cores n = 2048 takes 0.92 ms (3.80), 4096 2.66 (12.4), 8192 12.4 (47.3), 16384
+// 92.7 (230).
+int64_t compact_depth(int64_t n, size_t bytes) {
+    for (int64_t pb = PB; pb >= NB; pb /= 2)
+        if (compact_bytes(n, pb) <= bytes) return pb;
+    return 0;
 }
 
 // Scratch of the allocation-free entry point, sized for n <= REALQ_PREPARE_NOALLOC_MAX_N.
@@ -451,7 +468,7 @@ static realq_status_t prepare_steps(cudaStream_t s, int64_t n, float *U, float *
     return REALQ_OK;
 }
 
-// Wider inputs, 512 columns at a time.  Step K (block K = columns k0 .. k1):
+// Wider inputs, pb columns at a time.  Step K (block K = columns k0 .. k1):
 //   s      the cluster factors and inverts A[K, K] (in place: U_KK); the panel
 //          R[0:k0, K] = A[0:k0, K] U_KK^T; the update of the next block's
 //          columns, A[0:k0, K-1] -= R[0:k0, K] R[K-1, K]^T (upper)
@@ -461,20 +478,23 @@ static realq_status_t prepare_steps(cudaStream_t s, int64_t n, float *U, float *
 //          accumulated in place of R[I, j] (which step j consumed as planes):
 //            U[K, K+1:] = -U_KK S[K, K+1:], then for the rows I above
 //            S[I, K] = R[I, K] U_KK and S[I, K+1:] += R[I, K] U[K, K+1:].
-// So every product has depth 512 and as many tiles as the matrix gives it,
+// So every product has depth pb and as many tiles as the matrix gives it,
 // where one product per row block of U with a depth of up to n had few tiles
 // and a long chain.  A product's operands are three bf16 planes each.
+// compact: all of it on s, in compact_bytes of planes.
 static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *status, int *status_tc,
-                                      unsigned char *planes, bool overlap) {
+                                      unsigned char *planes, int64_t pb, bool compact, bool overlap) {
     Carve cv(planes);
-    auto take = [&](int64_t rows) { return cv.take<__nv_bfloat16>((size_t)rows * PB * 3); };
-    __nv_bfloat16 *Vp = take(PB), *Ap = take(n), *Rp[kPanels], *Sp, *Up;
-    for (int i = 0; i < kPanels; ++i) Rp[i] = take(n);
-    Sp = take(n);
-    Up = take(n);
-    const int nbk = ceil_div(n, PB);
+    auto take = [&](int64_t rows) { return cv.take<__nv_bfloat16>((size_t)rows * pb * 3); };
+    __nv_bfloat16 *Vp = take(pb), *Ap = take(n), *Rp[kPanels] = {Ap, Ap, Ap}, *Sp = nullptr, *Up = nullptr;
+    if (!compact) {
+        for (int i = 0; i < kPanels; ++i) Rp[i] = take(n);
+        Sp = take(n);
+        Up = take(n);
+    }
+    const int nbk = ceil_div(n, pb);
     AuxStream *aux = nullptr;
-    if (overlap) REALQ_TRY(aux_for(s, nbk, &aux));
+    if (overlap && !compact) REALQ_TRY(aux_for(s, nbk, &aux));
     cudaStream_t rs = aux ? aux->stream : s, wd = aux ? aux->wide : s;
     if (aux) {
         // the side streams follow everything already on s
@@ -482,15 +502,17 @@ static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *
         REALQ_CUDA_TRY(cudaStreamWaitEvent(rs, aux->ev[0], 0));
         REALQ_CUDA_TRY(cudaStreamWaitEvent(wd, aux->ev[0], 0));
     }
-    // planes of rows x PB terms, k terms of which exist
-    auto op = [&](const __nv_bfloat16 *p, int64_t rows, int64_t k) { return X6Planes{p, rows, k, PB, rows * PB}; };
+    // planes of rows x pb terms, k terms of which exist
+    auto op = [&](const __nv_bfloat16 *p, int64_t rows, int64_t k) { return X6Planes{p, rows, k, pb, rows * pb}; };
     for (int K = nbk - 1; K >= 0; --K) {
-        const int64_t k0 = (int64_t)K * PB, kb = std::min<int64_t>(PB, n - k0), k1 = k0 + kb, r = n - k1;
+        const int64_t k0 = (int64_t)K * pb, kb = std::min<int64_t>(pb, n - k0), k1 = k0 + kb, r = n - k1;
         __nv_bfloat16 *Rk = Rp[K % kPanels];
+        if (compact) Sp = Up = Ap + (size_t)k0 * pb * 3;
+        __nv_bfloat16 *Ukk = compact ? Vp : Up;   // U_KK for the row block's product
         REALQ_TRY(chol_inv_block(s, n, U + k0 * n + k0, kb, k0, status));
         if (k0 > 0) {
             // the planes of U_KK and of the panel, and the panel's solve (U_KK upper: terms k >= j)
-            const X6Split sv{U + k0 * n + k0, n, kb, kb, 0, Vp, PB, kb * PB}, sa{U + k0, n, k0, kb, 0, Ap, PB, k0 * PB};
+            const X6Split sv{U + k0 * n + k0, n, kb, kb, 0, Vp, pb, kb * pb}, sa{U + k0, n, k0, kb, 0, Ap, pb, k0 * pb};
             REALQ_TRY(split3(s, sa, &sv));
             X6Epi e{};
             e.mode = X6_STORE;
@@ -500,13 +522,13 @@ static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *
             REALQ_TRY(gemm_x6(s, op(Ap, k0, kb), op(Vp, kb, kb), k0, kb, kb, 0, 0, 0, 0, e, status_tc, "chol_panel_tc"));
             // (the planes that step K + kPanels left here are no longer read)
             if (aux && K + kPanels < nbk) REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->rdone[K + kPanels], 0));
-            const X6Split sr{U + k0, n, k0, kb, 0, Rk, PB, k0 * PB};
+            const X6Split sr{U + k0, n, k0, kb, 0, Rk, pb, k0 * pb};
             REALQ_TRY(split3(s, sr));
             if (aux) {
                 REALQ_CUDA_TRY(cudaEventRecord(aux->pdone[K], s));
                 REALQ_CUDA_TRY(cudaStreamWaitEvent(rs, aux->pdone[K], 0));
             }
-            const int64_t kw = k0 - PB;   // rows and columns of the wide part
+            const int64_t kw = k0 - pb;   // rows and columns of the wide part
             if (aux) REALQ_CUDA_TRY(cudaStreamWaitEvent(wd, aux->pdone[K], 0));
             // the narrow part's columns were last written by the wide part of step K + 1
             if (aux && K + 1 < nbk) REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->wdone[K + 1], 0));
@@ -515,7 +537,7 @@ static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *
             u.alpha = -1.f;
             u.C = U + kw; u.ldc = n;
             u.joff = kw;
-            REALQ_TRY(gemm_x6(s, op(Rk, k0, kb), op(Rk, k0, kb), k0, PB, kb, 0, kw, 0, 0, u, status_tc,
+            REALQ_TRY(gemm_x6(s, op(Rk, k0, kb), op(Rk, k0, kb), k0, pb, kb, 0, kw, 0, 0, u, status_tc,
                               "chol_update_tc"));
             if (kw > 0) {
                 X6Epi w{};
@@ -532,18 +554,19 @@ static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *
         }
         if (r > 0) {
             // U[K, K+1:] = -U_KK S[K, K+1:] (U_KK upper: terms k >= i)
-            const X6Split ss{U + k0 * n + k1, n, kb, r, 1, Sp, PB, r * PB}, sv{U + k0 * n + k0, n, kb, kb, 0, Up, PB, kb * PB};
-            REALQ_TRY(split3(rs, ss, &sv));
+            const X6Split ss{U + k0 * n + k1, n, kb, r, 1, Sp, pb, r * pb}, sv{U + k0 * n + k0, n, kb, kb, 0, Ukk, pb, kb * pb};
+            // (compact: above the last step the panel's solve has left them)
+            REALQ_TRY(split3(rs, ss, compact && k0 > 0 ? nullptr : &sv));
             X6Epi e{};
             e.mode = X6_STORE;
             e.C = U + k0 * n + k1; e.ldc = n;
             e.alpha = -1.f;
             e.a_lo = 1;
-            REALQ_TRY(gemm_x6(rs, op(Up, kb, kb), op(Sp, r, kb), kb, r, kb, 0, 0, 0, 0, e, status_tc, "trtri_panel_tc"));
+            REALQ_TRY(gemm_x6(rs, op(Ukk, kb, kb), op(Sp, r, kb), kb, r, kb, 0, 0, 0, 0, e, status_tc, "trtri_panel_tc"));
         }
         if (k0 > 0) {
             const int64_t rr = n - k0;
-            const X6Split su{U + k0 * n + k0, n, kb, rr, 1, Up, PB, rr * PB};
+            const X6Split su{U + k0 * n + k0, n, kb, rr, 1, Up, pb, rr * pb};
             REALQ_TRY(split3(rs, su));
             X6Epi e{};
             e.mode = X6_ADD;
@@ -568,6 +591,7 @@ realq_status_t prepare_impl(cudaStream_t s, int64_t n, double norm, float damp, 
     Carve cv(ws);
     int *status = cv.take<int>(1);
     float *lam = cv.take<float>(1);
+    const size_t rest = cv.off;
     float *Vd = cv.take<float>((size_t)NB * NB);
     float *panel = cv.take<float>(0);
     // status[0]: the failing column (-1: none); status[1]: timeout bits of
@@ -594,8 +618,10 @@ realq_status_t prepare_impl(cudaStream_t s, int64_t n, double norm, float damp, 
     if (n <= PB)
         REALQ_TRY(chol_inv_block(s, n, U, n, 0, status));
     else if (ws_bytes >= prepare_ws_bytes(n))
-        REALQ_TRY(prepare_blocked(s, n, U, status, status_tc, static_cast<unsigned char *>(ws) + prepare_bytes(n),
-                                  overlap));
+        REALQ_TRY(prepare_blocked(s, n, U, status, status_tc, static_cast<unsigned char *>(ws) + prepare_bytes(n), PB,
+                                  false, overlap));
+    else if (const int64_t pb = compact_depth(n, ws_bytes - rest))
+        REALQ_TRY(prepare_blocked(s, n, U, status, status_tc, static_cast<unsigned char *>(ws) + rest, pb, true, false));
     else
         REALQ_TRY(prepare_steps(s, n, U, Vd, panel, status));
     if (!sync) return REALQ_OK;  // the failing column stays in the workspace's first word
