@@ -207,7 +207,7 @@ struct DevExec {
             e.R = g.R; e.ldr = g.ldr;
             if (st == REALQ_OK)
                 st = gemm_x6(s, X6Planes{Ap, g.M, g.K, ldk, g.M * ldk}, X6Planes{Bp, g.N, g.K, ldk, g.N * ldk}, g.M, g.N,
-                             g.K, 0, 0, 0, 0, e, err, name);
+                             g.K, 0, e, err, name);
             return st != REALQ_OK;
         }
         if (tc_ok(g)) {
@@ -239,7 +239,6 @@ struct DevExec {
         a.C = g.C; a.ldc = g.ldc;
         a.R = g.R; a.ldr = g.ldr;
         a.alpha = g.alpha;
-        a.nsum = 1; a.nsum_b = 1; a.ksplit = 1;
         st = gemm_f32(s, g.a_kmajor ? A_KMAJOR : A_ROW, g.R ? EPI_BIAS : EPI_STORE, a, name);
         return st != REALQ_OK;
     }

@@ -61,7 +61,7 @@ struct X6Tile {
 template <int TN>
 __global__ void __launch_bounds__(THREADS, 1)
     gemm_x6_kernel(const __grid_constant__ CUtensorMap ma, const __grid_constant__ CUtensorMap mb, int64_t M, int64_t N,
-                   int64_t K, int a_row0, int b_row0, int a_k0, int b_k0, const X6Epi e, int *err) {
+                   int64_t K, int b_row0, const X6Epi e, int *err) {
     using TL = X6Tile<TN>;
     constexpr int STAGES = TL::STAGES;
     extern __shared__ uint8_t smem_raw[];
@@ -88,13 +88,12 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     if (e.mode == X6_UPPER && e.joff + j0 + TN <= i0) return;   // wholly below the diagonal (uniform over the CTA)
     // triangular operands shorten the K range: a_lo A(i, k) = 0 for k < i,
-    // b_lo B(j, k) = 0 for k < j, b_hi B(j, k) = 0 for k > j
-    int64_t kbeg = 0, kend = K;
+    // b_lo B(j, k) = 0 for k < j
+    int64_t kbeg = 0;
     if (e.a_lo && i0 > kbeg) kbeg = i0;
     if (e.b_lo && j0 > kbeg) kbeg = j0;
     kbeg = kbeg / KS * KS;
-    if (e.b_hi && kend > j0 + TN) kend = j0 + TN;
-    const int nk = kend > kbeg ? (int)((kend - kbeg + KS - 1) / KS) : 0;
+    const int nk = K > kbeg ? (int)((K - kbeg + KS - 1) / KS) : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -137,8 +136,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                 tc::mbar_arrive_expect_tx(fb, TL::STAGE_BYTES);
                 const int x = (int)kbeg + it * KS;
                 const uint32_t base = tc::smem_u32(smem + s * TL::STAGE_BYTES);
-                tc::tma_load_3d(base, &ma, fb, a_k0 + x, a_row0 + (int)i0, 0);
-                tc::tma_load_3d(base + NP * TL::PLANE_A, &mb, fb, b_k0 + x, b_row0 + (int)j0, 0);
+                tc::tma_load_3d(base, &ma, fb, x, (int)i0, 0);
+                tc::tma_load_3d(base + NP * TL::PLANE_A, &mb, fb, x, b_row0 + (int)j0, 0);
             }
             if (*abort_flag) {
                 int never = 0;
@@ -367,7 +366,7 @@ realq_status_t check_planes(const X6Planes &p, const char *name) {
 
 template <int TN>
 realq_status_t launch_x6(cudaStream_t s, const X6Planes &A, const X6Planes &B, int64_t M, int64_t N, int64_t K,
-                         int a_row0, int b_row0, int a_k0, int b_k0, const X6Epi &e, int *err) {
+                         int b_row0, const X6Epi &e, int *err) {
     CUtensorMap ma, mb;
     CUresult r = encode_tmap_3d_bf16(&ma, A.p, (uint64_t)A.k, (uint64_t)A.rows, NP, (uint64_t)A.ld * 2,
                                      (uint64_t)A.plane * 2, KS, TM, NP);
@@ -377,7 +376,7 @@ realq_status_t launch_x6(cudaStream_t s, const X6Planes &A, const X6Planes &B, i
     if (r != CUDA_SUCCESS) return fail(REALQ_ERR_CUDA, "cuTensorMapEncodeTiled (bf16 planes) failed (%d)", (int)r);
     REALQ_TRY(set_smem_limit(reinterpret_cast<const void *>(gemm_x6_kernel<TN>), X6Tile<TN>::SMEM));
     const dim3 grid((unsigned)ceil_div(N, TN), (unsigned)ceil_div(M, TM));
-    gemm_x6_kernel<TN><<<grid, THREADS, X6Tile<TN>::SMEM, s>>>(ma, mb, M, N, K, a_row0, b_row0, a_k0, b_k0, e, err);
+    gemm_x6_kernel<TN><<<grid, THREADS, X6Tile<TN>::SMEM, s>>>(ma, mb, M, N, K, b_row0, e, err);
     return REALQ_OK;
 }
 
@@ -398,13 +397,10 @@ realq_status_t split3(cudaStream_t s, const X6Split &a, const X6Split *b) {
 }
 
 realq_status_t gemm_x6(cudaStream_t s, const X6Planes &A, const X6Planes &B, int64_t M, int64_t N, int64_t K,
-                       int64_t a_row0, int64_t b_row0, int64_t a_k0, int64_t b_k0, const X6Epi &e, int *err,
-                       const char *name) {
+                       int64_t b_row0, const X6Epi &e, int *err, const char *name) {
     if (M <= 0 || N <= 0) return REALQ_OK;
     REALQ_TRY(check_planes(A, name));
     REALQ_TRY(check_planes(B, name));
-    if (a_k0 % 8 != 0 || b_k0 % 8 != 0)   // the x coordinate of every TMA box: 16-byte aligned
-        return fail(REALQ_ERR_INVALID_ARG, "%s: K offsets must be multiples of 8", name);
     // the 128 x 256 tile where it leaves no more of the last wave idle than it
     // saves in operand traffic (a 128 x 128 tile takes about 0.6 of its time)
     const int sms = num_sms();
@@ -413,9 +409,9 @@ realq_status_t gemm_x6(cudaStream_t s, const X6Planes &A, const X6Planes &B, int
     {
         Launch L(name, s);
         if (10 * w256 <= 6 * w128)
-            REALQ_TRY(launch_x6<256>(s, A, B, M, N, K, (int)a_row0, (int)b_row0, (int)a_k0, (int)b_k0, e, err));
+            REALQ_TRY(launch_x6<256>(s, A, B, M, N, K, (int)b_row0, e, err));
         else
-            REALQ_TRY(launch_x6<128>(s, A, B, M, N, K, (int)a_row0, (int)b_row0, (int)a_k0, (int)b_k0, e, err));
+            REALQ_TRY(launch_x6<128>(s, A, B, M, N, K, (int)b_row0, e, err));
     }
     return check_launch(name);
 }

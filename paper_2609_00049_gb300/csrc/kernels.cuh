@@ -34,16 +34,8 @@ struct GemmArgs {
     float *C; int64_t ldc;
     const float *R; int64_t ldr;
     float alpha;
-    // A_ROW only: A(i, k) = sum over s < nsum of A[s * aplane + i * lda + k]
-    int nsum; int64_t aplane;
-    // K split over gridDim.z; EPI_STORE writes slice z to C + z * cplane
-    int ksplit; int64_t cplane;
-    // A(i, k) = 0 for k < i: start each CTA's K range at its first row
-    int a_upper;
     // B(k, j) = 0 for k > j: end each CTA's K range at its last column
     int b_upper;
-    // B(k, j) = sum over s < nsum_b of B[s * bplane + k * ldb + j]
-    int nsum_b; int64_t bplane;
     // EPI_BGD_P operands
     const float *Ad; const float *Wc; const void *W0c; int w0_bf16;
     const uint8_t *dead; const float *lam; int64_t col0; int64_t ldw;
@@ -152,7 +144,7 @@ struct X6Epi {
     float *C; int64_t ldc;
     float alpha; const float *R; int64_t ldr;   // R: X6_STORE (nullable, may be C)
     int64_t joff, nstore;
-    int a_lo, b_lo, b_hi;                       // A(i, k) = 0 for k < i, B(j, k) = 0 for k < j, B(j, k) = 0 for k > j
+    int a_lo, b_lo;                             // A(i, k) = 0 for k < i, B(j, k) = 0 for k < j
 };
 // One operand to split into planes: src (rows x cols, row stride lds), as its
 // rows (dst[r * ldd + c]) or, with trans, its columns (dst[c * ldd + r]).
@@ -163,10 +155,9 @@ struct X6Split {
 };
 // one or two operands in one launch
 realq_status_t split3(cudaStream_t s, const X6Split &a, const X6Split *b = nullptr);
-// C (M x N) from rows a_row0.. of A and b_row0.. of B, K terms from a_k0 / b_k0 (multiples of 8) on
+// C (M x N) from the rows of A and the rows b_row0.. of B, K terms
 realq_status_t gemm_x6(cudaStream_t s, const X6Planes &A, const X6Planes &B, int64_t M, int64_t N, int64_t K,
-                       int64_t a_row0, int64_t b_row0, int64_t a_k0, int64_t b_k0, const X6Epi &e, int *err,
-                       const char *name);
+                       int64_t b_row0, const X6Epi &e, int *err, const char *name);
 
 // ------------------------------------------------- activation quantizer ---
 realq_status_t act_quant(cudaStream_t s, int64_t T, int64_t n, const void *X, realq_dtype_t dt, int bits, float a_clip,

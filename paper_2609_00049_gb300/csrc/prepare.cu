@@ -415,7 +415,6 @@ realq_status_t prepare_deferred(cudaStream_t s, int64_t n, double norm, float da
 //   U[K, K] = R_KK^-1,  U[K, K+1:] = -U[K, K] (R[K, K+1:] U[K+1:, K+1:])
 // (after step K no later step reads row block K of R).
 static realq_status_t prepare_steps(cudaStream_t s, int64_t n, float *U, float *Vd, float *panel, int *status) {
-    const int64_t plane = n * NB;
     const int nbk = ceil_div(n, NB);
     for (int K = nbk - 1; K >= 0; --K) {
         const int64_t k0 = (int64_t)K * NB;
@@ -452,14 +451,14 @@ static realq_status_t prepare_steps(cudaStream_t s, int64_t n, float *U, float *
             g.A = U + k0 * n + k1; g.lda = n;
             g.B = U + k1 * n + k1; g.ldb = n;
             g.C = panel; g.ldc = n;
-            g.cplane = plane; g.b_upper = 1;
+            g.b_upper = 1;
             g.alpha = 1.f;
             REALQ_TRY(gemm_f32(s, A_ROW, EPI_STORE, g, "trtri_trmm"));
             // U[K, K+1:] = -U_KK X, U_KK read from A[K, K] (upper, zeros below)
             GemmArgs h{};
             h.M = kb; h.N = r; h.K = kb;
             h.A = U + k0 * n + k0; h.lda = n;
-            h.B = panel; h.ldb = n; h.nsum_b = 1; h.bplane = plane;
+            h.B = panel; h.ldb = n;
             h.C = U + k0 * n + k1; h.ldc = n;
             h.alpha = -1.f;
             REALQ_TRY(gemm_f32(s, A_ROW, EPI_STORE, h, "trtri_panel"));
@@ -519,7 +518,7 @@ static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *
             e.C = U + k0; e.ldc = n;
             e.alpha = 1.f;
             e.b_lo = 1;
-            REALQ_TRY(gemm_x6(s, op(Ap, k0, kb), op(Vp, kb, kb), k0, kb, kb, 0, 0, 0, 0, e, status_tc, "chol_panel_tc"));
+            REALQ_TRY(gemm_x6(s, op(Ap, k0, kb), op(Vp, kb, kb), k0, kb, kb, 0, e, status_tc, "chol_panel_tc"));
             // (the planes that step K + kPanels left here are no longer read)
             if (aux && K + kPanels < nbk) REALQ_CUDA_TRY(cudaStreamWaitEvent(s, aux->rdone[K + kPanels], 0));
             const X6Split sr{U + k0, n, k0, kb, 0, Rk, pb, k0 * pb};
@@ -537,14 +536,14 @@ static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *
             u.alpha = -1.f;
             u.C = U + kw; u.ldc = n;
             u.joff = kw;
-            REALQ_TRY(gemm_x6(s, op(Rk, k0, kb), op(Rk, k0, kb), k0, pb, kb, 0, kw, 0, 0, u, status_tc,
+            REALQ_TRY(gemm_x6(s, op(Rk, k0, kb), op(Rk, k0, kb), k0, pb, kb, kw, u, status_tc,
                               "chol_update_tc"));
             if (kw > 0) {
                 X6Epi w{};
                 w.mode = X6_UPPER;
                 w.alpha = -1.f;
                 w.C = U; w.ldc = n;
-                REALQ_TRY(gemm_x6(wd, op(Rk, k0, kb), op(Rk, k0, kb), kw, kw, kb, 0, 0, 0, 0, w, status_tc,
+                REALQ_TRY(gemm_x6(wd, op(Rk, k0, kb), op(Rk, k0, kb), kw, kw, kb, 0, w, status_tc,
                                   "chol_update_tc"));
             }
             if (aux) REALQ_CUDA_TRY(cudaEventRecord(aux->wdone[K], wd));
@@ -562,7 +561,7 @@ static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *
             e.C = U + k0 * n + k1; e.ldc = n;
             e.alpha = -1.f;
             e.a_lo = 1;
-            REALQ_TRY(gemm_x6(rs, op(Ukk, kb, kb), op(Sp, r, kb), kb, r, kb, 0, 0, 0, 0, e, status_tc, "trtri_panel_tc"));
+            REALQ_TRY(gemm_x6(rs, op(Ukk, kb, kb), op(Sp, r, kb), kb, r, kb, 0, e, status_tc, "trtri_panel_tc"));
         }
         if (k0 > 0) {
             const int64_t rr = n - k0;
@@ -573,7 +572,7 @@ static realq_status_t prepare_blocked(cudaStream_t s, int64_t n, float *U, int *
             e.alpha = 1.f;
             e.C = U + k0; e.ldc = n;
             e.nstore = kb;
-            REALQ_TRY(gemm_x6(rs, op(Rk, k0, kb), op(Up, rr, kb), k0, rr, kb, 0, 0, 0, 0, e, status_tc, "trtri_update_tc"));
+            REALQ_TRY(gemm_x6(rs, op(Rk, k0, kb), op(Up, rr, kb), k0, rr, kb, 0, e, status_tc, "trtri_update_tc"));
             if (aux) REALQ_CUDA_TRY(cudaEventRecord(aux->rdone[K], rs));
         }
     }
