@@ -19,8 +19,13 @@
 // about 1 - 5e-8 on every output, which the window's difference of two passes
 // does not average out as it does a random one (a window sweep's group scales
 // moved by 2e-6 instead of 3e-7).  Three slices of every eight are therefore
-// added with the factor 1 + 2^-23, which is the expected loss: the mean error
-// is then within 0.3e-8 of the output's scale.
+// added with the factor 1 + 2^-23, which is the expected loss of dense random
+// terms: with K a multiple of 256 their mean error is within 0.3e-8 of the
+// output's scale.  It is not a bound for every operand: a product of one slice
+// (K <= 32) keeps its -4.5e-8, one of two (K = 64) is left with +1.5e-8, a sum
+// that one slice holds nearly all of (sparse or diagonal operands) takes that
+// slice's -5e-8 or +1.2e-7, and sums of small integers, which the slices form
+// exactly, are moved by up to one unit in the last place.
 //
 // One CTA owns a 128 x TN tile (TN = 256, or 128 where that fills the SMs
 // better): warp 8 issues the TMA loads (one 3-D box per operand and stage: 32
@@ -271,7 +276,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 // The three bf16 parts of v, rounded to nearest (a finite value whose first
 // part would round to infinity is truncated instead; the parts of a
 // non-finite value are the value and zeros, so that a product with an infinite
-// operand is infinite or, where the other's later parts are zero, NaN).
+// operand is not finite: infinite where the other's three parts have one sign
+// and none is zero, else NaN, where the fp32 product gives infinity).
 __device__ __forceinline__ void split3(float v, __nv_bfloat16 &a, __nv_bfloat16 &b, __nv_bfloat16 &c) {
     a = __float2bfloat16_rn(v);
     float h = __bfloat162float(a);

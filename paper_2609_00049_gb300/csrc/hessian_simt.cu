@@ -293,6 +293,10 @@ realq_status_t hessian_reduce(cudaStream_t s, int64_t n, int splits, const float
     return check_launch("hessian_reduce");
 }
 
+// The CUDA-core kernels' token splits, with and without D and for both tile
+// sizes (so that all take the same sums): by the 128-channel row blocks times the
+// 256-channel column blocks that reach the diagonal, about half of the 128 x 128
+// tiles, so that up to twice as many CTAs as SMs start.
 int hessian_splits(int64_t n, int64_t T, int sms) {
     const int nti = ceil_div(n, 128);
     int64_t tiles = 0;

@@ -67,10 +67,10 @@ constexpr int KSTAGE = 64;                       // tokens per pipeline stage
 constexpr int STAGES = 6;
 // 512 tokens per TMEM accumulator pass, with and without D: H then has the same
 // bits whether or not D is asked for.  D, the small difference of two large
-// sums, magnifies the accumulator's rounding and sets the length (n = 2056, T =
-// 50,001: 690 us and 5e-6 to 7e-6 of D's scale against 64 bits; with 1024 tokens
-// 636 us and 9e-6 to 11e-6).  H alone takes 6 % longer for it, at half the error:
-// n = 8192, T = 65,536: 3.07 -> 3.26 ms, 2.2e-6 -> 1.1e-6.
+// sums, magnifies the accumulator's rounding and sets the length: n = 2056, T =
+// 50,001 5e-6 to 7e-6 of D's scale against 64 bits, with 1024 tokens 9e-6 to
+// 11e-6.  (n = 8192, T = 65,536 takes 3.02 ms and 1.0e-6, with 1024 tokens and
+// spilled registers it took 3.07 ms and 2.2e-6.)
 constexpr int CHUNK_STAGES = 8;
 constexpr int DRAIN_WARPS = 8;                   // two per TMEM lane quarter, 128 columns each
 constexpr int THREADS = (DRAIN_WARPS + 2) * 32;  // + the TMA warp and the MMA warp
@@ -557,13 +557,15 @@ bool hessian_tc_eligible(int64_t n, int64_t T, const void *X) {
            n < (1ll << 31);
 }
 
-// Token splits of a launch of full (and 0.35 of a full one's time: last-block)
-// tiles over the pairs of SMs: the count that minimises rounds x (a split's
-// share of a tile's time + a CTA's fixed cost) + the partial sums' traffic,
-// in microseconds (a 64-token stage of a pair is 0.29 us at 1.75 GHz; a CTA's
-// start, fill and epilogue about 8 us; a partial 256 x 256 tile written and
-// read at 5 TB/s).  At least 1024 tokens per split (two accumulator passes) and at
-// most 16 splits.
+// Token splits of a launch of full (and, as 0.35 of one, last-block) tiles over
+// the pairs of SMs: the count that minimises rounds x (a split's share of a
+// tile's time + a CTA's fixed cost) + the partial sums' traffic, in microseconds
+// (a 64-token stage of a pair is 0.29 us at 1.75 GHz; a CTA's start, fill and
+// epilogue about 8 us; a partial 256 x 256 tile written and read at 5 TB/s).  0.35
+// is the time of a last block of 8 channels; a wide one (n % 256 near 256) takes
+// up to a full tile's time, which the count then undercharges (n = 2040, T =
+// 50,001 takes 197 us so, against 344 on the kernel before the pairs).  At least
+// 1024 tokens per split (two accumulator passes) and at most 16 splits.
 static int tc_splits(const HessGrid &g, int64_t T, int sms) {
     const int64_t full = (g.nsym ? (int64_t)g.nf * (g.nf + 1) / 2 : 0) + (g.ncross ? (int64_t)g.nf * g.nf : 0);
     const double tiles = (double)full + 0.35 * (double)(g.nsym + g.ncross - full);
