@@ -20,7 +20,7 @@
 // last place per accumulated MMA, in one direction, so a TMEM accumulator that
 // takes all 2^18 tokens of a calibration set (2^14 MMAs) drifts by ~1e-3 of
 // the entry.  The accumulation is therefore promoted: TMEM holds two 128 x 256
-// accumulators (per CTA), the MMA issuer switches between them every 512 tokens
+// accumulators (per CTA), the MMA issuer switches between them every 640 tokens
 // (CHUNK_STAGES), and the eight drain warps add each finished chunk into fp32
 // registers (IEEE adds) while the other accumulator fills.
 //
@@ -65,13 +65,14 @@ constexpr int TM = 128;                          // tile rows of one CTA (channe
 constexpr int TN = 256;                          // tile rows of the pair, and tile columns (channels j)
 constexpr int KSTAGE = 64;                       // tokens per pipeline stage
 constexpr int STAGES = 6;
-// 512 tokens per TMEM accumulator pass, with and without D: H then has the same
+// 640 tokens per TMEM accumulator pass, with and without D: H then has the same
 // bits whether or not D is asked for.  D, the small difference of two large
-// sums, magnifies the accumulator's rounding and sets the length: n = 2056, T =
-// 50,001 5e-6 to 7e-6 of D's scale against 64 bits, with 1024 tokens 9e-6 to
-// 11e-6.  (n = 8192, T = 65,536 takes 3.02 ms and 1.0e-6, with 1024 tokens and
-// spilled registers it took 3.07 ms and 2.2e-6.)
-constexpr int CHUNK_STAGES = 8;
+// sums, magnifies the accumulator's rounding and sets the length: it is the
+// longest with which D's error against 64 bits (2-norm, mean over 6 to 14 seeds) is
+// no larger at any measured shape than with one CTA per tile and 1024 tokens.
+// n = 2056, T = 50,001: 8.5e-6 so; here 512 tokens 6.3e-6, 640 7.3e-6, 704 8.9e-6,
+// 1024 8.7e-6.  n = 1024, T = 65,536: 8.3e-6; 4.2e-6, 5.1e-6, 6.6e-6, 7.3e-6.
+constexpr int CHUNK_STAGES = 10;
 constexpr int DRAIN_WARPS = 8;                   // two per TMEM lane quarter, 128 columns each
 constexpr int THREADS = (DRAIN_WARPS + 2) * 32;  // + the TMA warp and the MMA warp
 constexpr int BOX_BYTES = 64 * KSTAGE * 2;       // one TMA box (64 channels x 64 tokens)
@@ -565,7 +566,7 @@ bool hessian_tc_eligible(int64_t n, int64_t T, const void *X) {
 // is the time of a last block of 8 channels; a wide one (n % 256 near 256) takes
 // up to a full tile's time, which the count then undercharges (n = 2040, T =
 // 50,001 takes 197 us so, against 344 on the kernel before the pairs).  At least
-// 1024 tokens per split (two accumulator passes) and at most 16 splits.
+// 1024 tokens per split and at most 16 splits.
 static int tc_splits(const HessGrid &g, int64_t T, int sms) {
     const int64_t full = (g.nsym ? (int64_t)g.nf * (g.nf + 1) / 2 : 0) + (g.ncross ? (int64_t)g.nf * g.nf : 0);
     const double tiles = (double)full + 0.35 * (double)(g.nsym + g.ncross - full);

@@ -27,7 +27,7 @@ namespace {
 constexpr int SEL_THREADS = 1024;
 // Saliency spreads token magnitudes over decades, so a TMEM accumulator loses
 // the low bits of small terms against a running sum dominated by a few large
-// ones; promote to fp32 registers every 2 stages (128 tokens) instead of 8.
+// ones; promote to fp32 registers every 2 stages (128 tokens) instead of 10.
 constexpr int kPromoteStages = 2;
 
 __device__ __forceinline__ uint32_t key_of(float v) { return __float_as_uint(fmaxf(v, 0.f)); }
