@@ -4,7 +4,7 @@
 // and the updates of the blocked Cholesky / triangular inverse.
 //
 // C tile BM x BN per CTA (128 x 128, or 64 x 64 when the 128-tile grid would
-// leave most SMs idle), 256 threads, K staged 16 at a time through two
+// leave most SMs idle or M is at most 64), 256 threads, K staged 16 at a time through two
 // shared-memory buffers: the next K slice is loaded into registers while the
 // current one is multiplied, so global latency overlaps the FFMA work.
 #include "kernels.cuh"
@@ -163,7 +163,9 @@ void launch_epi(cudaStream_t s, EpiMode em, const GemmArgs &g, dim3 grid) {
 template <int AM>
 realq_status_t dispatch(cudaStream_t s, EpiMode em, const GemmArgs &g, const char *name) {
     const int64_t big_tiles = (int64_t)ceil_div(g.N, 128) * ceil_div(g.M, 128);
-    const bool small = big_tiles < num_sms();
+    // 64 x 64 tiles also where a large one would be half empty (64 rows by 24,512
+    // columns and as deep, a preparation's step: 803 against 659 ms over n = 24,576)
+    const bool small = big_tiles < num_sms() || g.M <= 64;
     {
         Launch L(name, s);
         if (small) launch_epi<64, 64, AM>(s, em, g, dim3(ceil_div(g.N, 64), ceil_div(g.M, 64)));
