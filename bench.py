@@ -47,9 +47,9 @@ NCU_TRAFFIC = {
     # average launch (1.995 TFLOP)
     ("llama3.1-70b", "bgd_p_gemm"): 6584000000,
     # the four Hessians of one step of the same block, one-pass counters:
-    # down_in (n = 28,672) 1010 GB, the three n = 8192 inputs 58-66 GB each;
+    # down_in (n = 28,672) 1592 GB, the three n = 8192 inputs 67-91 GB each;
     # averaged per launch
-    ("llama3.1-70b", "hessian_syrk_tc"): 299400000000,
+    ("llama3.1-70b", "hessian_syrk_tc"): 455100000000,
 }
 
 
@@ -370,7 +370,9 @@ def work_models(wl, args=None):
         per_step["saliency_scale"] = ("hbm", sum(wl.inputs[md.input].T * md.n * 6 * ng for md in wl.modules),
                                       "GB/s")
     if getattr(args, "act_bits", 0):
-        # D = X̂ᵀX̂ - XᵀX̂: the full non-symmetric product XᵀX̂ per input
+        # D = X̂ᵀX̂ - XᵀX̂: the full non-symmetric product XᵀX̂ per input (a launch
+        # of its own without token splits; with splits hessian_syrk_tc's launch
+        # does both products, and its rate above counts the symmetric one only)
         per_step["hessian_cross_tc"] = ("tensor", sum(2 * s.T * s.n * s.n for s in wl.inputs.values()), "TFLOP/s")
         per_step["act_quant"] = ("hbm", sum(s.T * s.n * 2 * 3 for s in wl.inputs.values()), "GB/s")
     bgd_p = bgd_g = trail = trail_planes = 0
@@ -422,13 +424,13 @@ def work_models(wl, args=None):
     per_step["bgd_g_gemm_adam"] = ("f16x3" if f16 else "tf32x3", bgd_g, "TFLOP/s")
     if f16:
         # the step's and P^T's fp16 planes, per block: read the fp32 values
-        # twice (row maximum, then split) and write two 2-byte planes
+        # and write two 2-byte planes
         f16_split = 0
         for md in wl.modules:
             m, n, B = md.m, md.n, wl.block_size
             for b in range(-(-n // B)):
                 r = n - min((b + 1) * B, n)
-                f16_split += 12 * m * (n - b * B) * (b > 0) + 12 * m * r
+                f16_split += 8 * m * (n - b * B) * (b > 0) + 8 * m * r
         per_step["f16_split"] = ("hbm", f16_split, "GB/s")
     per_step["trailing_update"] = ("tf32x3", trail, "TFLOP/s")
     per_step["trailing_planes"] = ("hbm", trail_planes, "GB/s")
