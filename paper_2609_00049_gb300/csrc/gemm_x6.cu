@@ -93,10 +93,10 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     if (e.mode == X6_UPPER && e.joff + j0 + TN <= i0) return;   // wholly below the diagonal (uniform over the CTA)
     // triangular operands shorten the K range: a_lo A(i, k) = 0 for k < i,
-    // b_lo B(j, k) = 0 for k < j
-    int64_t kbeg = 0;
-    if (e.a_lo && i0 > kbeg) kbeg = i0;
-    if (e.b_lo && j0 > kbeg) kbeg = j0;
+    // b_lo B(j, k) = 0 for k < j (32 bits hold it: the operands' k is checked)
+    int kbeg = 0;
+    if (e.a_lo && i0 > kbeg) kbeg = (int)i0;
+    if (e.b_lo && j0 > kbeg) kbeg = (int)j0;
     kbeg = kbeg / KS * KS;
     const int nk = K > kbeg ? (int)((K - kbeg + KS - 1) / KS) : 0;
 
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
                 const uint32_t fb = tc::smem_u32(&full[s]);
                 tc::mbar_arrive_expect_tx(fb, TL::STAGE_BYTES);
-                const int x = (int)kbeg + it * KS;
+                const int x = kbeg + it * KS;
                 const uint32_t base = tc::smem_u32(smem + s * TL::STAGE_BYTES);
                 tc::tma_load_3d(base, &ma, fb, x, (int)i0, 0);
                 tc::tma_load_3d(base + NP * TL::PLANE_A, &mb, fb, x, b_row0 + (int)j0, 0);
